@@ -205,7 +205,8 @@ typedef struct aeb_job_stats {
 
 /* Launch shape of the rollout kernels (chosen by aeb_autotune or set). */
 typedef struct aeb_launch_config {
-    int32_t tile;           /* samples per warp tile: 32..256, multiple of 32   */
+    int32_t tile;           /* samples per warp tile: 32..256, multiple of 32
+                               (32 in use until one is set or tuned)            */
     int32_t blocks_per_sm;  /* resident blocks per SM (0: as many as fit)       */
 } aeb_launch_config;
 

@@ -75,7 +75,7 @@ extern "C" aeb_status aeb_batch_create(const aeb_model *model, const aeb_job *jo
         return fail(AEB_EINVAL, "aeb_batch_create: stats is not 8-byte aligned");
 
     const LaunchCfg cfg = launch_cfg(precision);
-    const uint32_t T = (uint32_t)cfg.tile;
+    const uint32_t T = ticket_tile(cfg);
     std::vector<JobDev> hj(n_jobs);
     std::vector<TileDesc> tiles, red;
     std::vector<uint32_t> first(n_jobs + 1);
@@ -221,6 +221,7 @@ extern "C" aeb_status aeb_set_launch_config(aeb_precision precision, const aeb_l
     LaunchCfg c = launch_cfg(precision);
     c.tile = cfg->tile;
     c.blocks_per_sm = cfg->blocks_per_sm;
+    c.tile_set = true;
     set_launch_cfg(precision, c);
     return AEB_OK;
 }
@@ -295,8 +296,7 @@ extern "C" aeb_status aeb_autotune(const aeb_model *model, const aeb_params *par
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return fail(AEB_ECUDA, "aeb_autotune: cudaEventCreate failed");
     const LaunchCfg saved = launch_cfg(precision);
-    const int tiles64[] = {64, 128, 256}, tiles32[] = {32, 64, 128};
-    const int *tl = precision == AEB_FP64_PLAIN ? tiles64 : tiles32;
+    const int tl[] = {32, 64, 128};
     float best_ms = 1e30f;
     aeb_launch_config win{saved.tile, saved.blocks_per_sm};
     for (int ti = 0; ti < 3 && st == AEB_OK; ++ti) {
@@ -304,6 +304,7 @@ extern "C" aeb_status aeb_autotune(const aeb_model *model, const aeb_params *par
             LaunchCfg c = saved;
             c.tile = tl[ti];
             c.blocks_per_sm = bps;
+            c.tile_set = true;
             set_launch_cfg(precision, c);
             float ms = 0.0f;
             for (int rep = 0; rep < 2 && st == AEB_OK; ++rep) {  // warm-up, then timed

@@ -197,7 +197,7 @@ aeb_status scratch_for(cudaStream_t s, size_t bytes, void **out)
 }
 
 std::mutex g_cfg_mu;
-LaunchCfg g_cfg[2] = {{128, 0, 256}, {128, 0, 32}};
+LaunchCfg g_cfg[2] = {{128, 0, 256, false}, {128, 0, 32, false}};
 
 aeb_status rollout_impl(const ModelDev &md, const ParamsDev &pd, uint64_t n,
                         aeb_precision precision, const OutDev &od, cudaStream_t s,
@@ -210,7 +210,7 @@ aeb_status rollout_impl(const ModelDev &md, const ParamsDev &pd, uint64_t n,
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(counter)");
     const LaunchCfg cfg = launch_cfg(precision);
-    WorkDev w{n, (uint32_t)cfg.tile, counter, nullptr, 0, nullptr, key_base};
+    WorkDev w{n, ticket_tile(cfg), counter, nullptr, 0, nullptr, key_base};
     e = (precision == AEB_FP64_PLAIN) ? launch_rollout_fp64(md, pd, od, w, cfg, s)
                                       : launch_rollout_fp32(md, pd, od, w, cfg, s);
     if (e != cudaSuccess) return cuda_fail(e, "rollout launch");

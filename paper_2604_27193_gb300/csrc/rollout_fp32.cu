@@ -65,7 +65,6 @@
 namespace aeb {
 namespace {
 
-constexpr int kTileDefault = 32;  // samples per warp tile unless configured
 constexpr int kTileMax = 256;
 constexpr int kWarps = 4;      // warps per block
 constexpr int kThreads = 32 * kWarps;
@@ -1375,7 +1374,7 @@ cudaError_t launch_t(const ModelDev &m, const ParamsDev &p, const OutDev &o, con
                      const LaunchCfg &cfg, cudaStream_t s)
 {
     auto kern = k_rollout_fp32<LEAD, TTC, PERC>;
-    const int T = w.tiles ? (int)w.tile : (cfg.tile > 0 ? cfg.tile : kTileDefault);
+    const int T = (int)w.tile;
     if (T < 32 || T > kTileMax || T % 32) return cudaErrorInvalidValue;
     const size_t smem = smem_per_block<TTC, PERC>(T);
     int dev = 0, sms = 0, per_sm = cfg.blocks_per_sm;

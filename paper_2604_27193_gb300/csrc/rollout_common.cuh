@@ -188,46 +188,3 @@ __device__ __forceinline__ void load_fields(const ParamsDev &p, uint64_t i, doub
 }
 
 }  // namespace aeb
-
-namespace aeb {
-
-// The per-warp driver shared by both precisions.  `Lane` provides
-//   bool init(M, X, P, O, p, o, k, thr) -- load parameter row p (output row o,
-//                                perception key row k); true if it already ended
-//   bool step(M, X, P, O, i)  -- one RK4 step; true if the rollout ended (stored)
-// where X holds precision-specific constants (kernel parameters, so the
-// compiler reads them from the parameter bank rather than registers).
-// Each lane owns one rollout at a time (Sec. V-A, one thread per sample); a
-// lane whose rollout ends takes the next sample of its warp's tile, so a warp
-// keeps all 32 lanes busy until the tiles run out instead of idling until its
-// slowest rollout ends.  There is no wait on other warps or on the host: the
-// loop ends when no lane holds a rollout.
-template <class Lane, class X>
-__device__ __forceinline__ void rollout_driver(const ModelDev &M, const X &Xc, const ParamsDev &P,
-                                               const OutDev &O, const WorkDev &W, uint32_t tile_size)
-{
-    const unsigned lane = threadIdx.x & 31u;
-    WarpQueue q;
-    Lane L;
-    uint64_t pidx = 0, oidx = 0, kidx = 0;
-    double thr = M.ttc_thr;
-    bool active = false;
-    unsigned need = kFull;
-    for (;;) {
-        while (need) {
-            const bool got = q.take(need, W, tile_size, M.ttc_thr, pidx, oidx, kidx, thr);
-            bool ended = false;
-            if ((need >> lane) & 1u) {
-                active = got;
-                if (active) ended = L.init(M, Xc, P, O, pidx, oidx, kidx, thr);
-            }
-            need = __ballot_sync(kFull, ended);
-        }
-        if (!__any_sync(kFull, active)) return;
-        bool ended = false;
-        if (active) ended = L.step(M, Xc, P, O, oidx);
-        need = __ballot_sync(kFull, ended);
-    }
-}
-
-}  // namespace aeb

@@ -20,6 +20,18 @@
 // and the fourth the largest when dt / tau <= 2), each stage evaluates only
 // that line, with the same expression as the full minimum, and the result
 // is the same bits.  Other steps evaluate the full minimum and re-select.
+//
+// What bounds it.  An SM sub-partition's binary64 unit holds a warp
+// instruction for 64 cycles if it is a fused multiply-add of three register
+// operands and for 76 otherwise (an add, a multiply, an immediate or constant
+// operand), whatever the number of warps, chains or busy lanes.  So inside a
+// piece every operation is written as a fused multiply-add of registers that
+// rounds to the same bits: a + b is fma(a, 1, b), a b is fma(a, b, -0), and
+// v + 2 w is fma(2, w, v), since doubling is exact away from overflow (a lane
+// takes this path only while its state is far inside the normal range, see
+// `tame`); the constants 1, 2, -0, dt and its fractions are kept in registers
+// the compiler cannot take for constants.  51 operations of 64 cycles a step
+// (59 on an axle line) against 57 (65) of 76.
 #include <climits>
 
 #include "rollout_common.cuh"
@@ -58,7 +70,38 @@ __device__ __forceinline__ long long okey(double x)
     return b < 0 ? -(b & 0x7fffffffffffffffll) : b;
 }
 
-struct NoExtra {};
+// int_to_double(n) for n >= 0, exact, on the integer pipe.
+__device__ __forceinline__ double from_int(int32_t n)
+{
+    if (n <= 0) return 0.0;
+    const int e = 31 - __clz(n);
+    const long long m = (long long)n << (52 - e);  // implicit one at bit 52
+    return __longlong_as_double(m + ((long long)(1022 + e) << 52));
+}
+
+// Step constants in registers, and the operations of a step as fused
+// multiply-adds of register operands (the same bits as the plain operation).
+struct Ops {
+    double one, two, nz, dt, h2, h6;
+    __device__ __forceinline__ double add(double a, double b) const { return __fma_rn(a, one, b); }
+    __device__ __forceinline__ double sub(double a, double b) const { return __fma_rn(b, -one, a); }
+    __device__ __forceinline__ double mul(double a, double b) const { return __fma_rn(a, b, nz); }
+    // a + 2 b, where 2 b does not overflow
+    __device__ __forceinline__ double add2(double a, double b) const { return __fma_rn(two, b, a); }
+    // h6 (((a + 2 b) + 2 c) + d) + y, rounded after each operation of the definition
+    __device__ __forceinline__ double combine(double y, double a, double b, double c, double d) const
+    {
+        return add(y, mul(h6, add(add2(add2(a, b), c), d)));
+    }
+};
+
+// Bounds of the states the fused forms are used on: they keep every sum and
+// product of a step below 2^400, so nothing overflows.
+constexpr double kTame = 1e5;
+__device__ __forceinline__ bool tame_speed(double v)  // 0 < v < ~1e5 (false for a NaN)
+{
+    return (unsigned)__double2hiint(v) < 0x40f86a00u;
+}
 
 __device__ __forceinline__ double dinf() { return __longlong_as_double(0x7ff0000000000000ll); }
 
@@ -87,6 +130,7 @@ struct Lane64 {
     int32_t n, n_b, n_delay;
     int piece;                    // 0: D, 1, 2: an axle line, 3: the constant cap; -1: none
     bool trig, lagged, ordered;
+    bool active;                  // the lane holds a rollout
 
     // Select the line that is the strict minimum at demand D and the demand
     // interval, shrunk by the band, on which it stays so (piece -1 if D is
@@ -122,6 +166,7 @@ struct Lane64 {
             else lo = fmax(lo, B + band);
         }
         if (!(lo <= D && D <= hi)) return;
+        if (!(fabs(A[cur]) < 1e50 && fabs(S[cur]) < 1e50)) return;  // see Ops
         klo = okey(lo);
         khi = okey(hi);
         if (CAP == AEB_CAP_LUMPED) {
@@ -135,13 +180,17 @@ struct Lane64 {
 
     // dv/dt on the current piece: the same value as `accel` for D in the
     // piece's interval.  `lines`: some lane of the warp is on an axle line.
-    __device__ __forceinline__ double accel_piece(double vv, double aa, bool lines) const
+    __device__ __forceinline__ double accel_piece(const Ops &q, double vv, double aa,
+                                                  bool lines) const
     {
         const double D = -aa;
         const double c = (CAP == AEB_CAP_LUMPED) ? cap : mg;
         double r = (piece == 0) ? D : c;
-        if (CAP != AEB_CAP_LUMPED && lines && (piece == 1 || piece == 2)) r = pa + pb * D;
-        return ((-r) - (k * vv) * vv) - gs;
+        if (CAP != AEB_CAP_LUMPED && lines) {
+            const double rl = q.add(pa, q.mul(pb, D));
+            if (piece == 1 || piece == 2) r = rl;
+        }
+        return q.sub(q.sub(-r, q.mul(q.mul(k, vv), vv)), gs);
     }
 
     // Realised deceleration r for demand D = -a (Eq. 5 as printed, or the
@@ -166,7 +215,7 @@ struct Lane64 {
         return TTC ? (trig ? n_b : -1) : n_delay;
     }
 
-    __device__ __forceinline__ bool init(const ModelDev &M, const NoExtra &, const ParamsDev &P,
+    __device__ __forceinline__ bool init(const ModelDev &M, const ParamsDev &P,
                                          const OutDev &O, uint64_t pi, uint64_t i, uint64_t ki,
                                          double thr_job)
     {
@@ -185,7 +234,9 @@ struct Lane64 {
         k = ((M.rho * f[kCd]) * M.area) / (2.0 * f[kMass]);
         lagged = f[kTau] > 0.0;
         it = lagged ? 1.0 / f[kTau] : 0.0;
-        ordered = !lagged || M.dt * it <= 2.0;
+        // (and the sample is inside the range of the fused forms)
+        ordered = (!lagged || M.dt * it <= 2.0) && M.dt >= 1e-30 && M.dt <= 1.0 &&
+                  fabs(M.a_cmd) <= kTame && k <= 1.0 && fabs(gs) <= kTame;
         const double mu = f[kMu], gc = f[kGc];
         const double mh = mu * M.hl;
         if (CAP == AEB_CAP_LUMPED) {
@@ -221,48 +272,54 @@ struct Lane64 {
         return false;
     }
 
-    __device__ __forceinline__ bool step(const ModelDev &M, const NoExtra &, const ParamsDev &,
-                                         const OutDev &O, uint64_t i)
+    // TTC trigger (while not yet triggered), at the start of step n.
+    __device__ __forceinline__ void test_trigger(const ModelDev &M, const Ops &q)
     {
-        const double dt = M.dt, h2 = M.h2, h6 = M.h6;
-        if (TTC && !trig) {
-            double gap_meas, closing;
-            if (M.lead_moving) {  // gap and closing speed to the moving lead
-                const double t = (double)n * dt;
-                gap_meas = ((d0 + lead_pos(M, t)) - x) + noise;
-                closing = v - lead_speed(M, t);
-            } else {
-                gap_meas = (d0 - x) + noise;
-                closing = v;
-            }
-            bool reading = true;
-            if (M.perc) {  // the reading of step n + L describes step n
-                uint32_t h[4];
-                perc_halves(row, (uint64_t)((long long)n + M.perc_lat), M.perc_seed, h);
-                const double s32 = 1.0 / 4294967296.0;  // 2^-32
-                const double u1 = (double)h[0] * s32, u2 = (double)h[1] * s32;
-                const double u3 = (double)h[2] * s32, u4 = (double)h[3] * s32;
-                if (u4 < M.perc_drop) reading = false;
-                else gap_meas = gap_meas + M.perc_sigma * (2.0 * (((u1 + u2) + u3) - 1.5));
-            }
-            if (reading && gap_meas <= thr * closing) {
-                trig = true;
-                long long nb = ((long long)n + M.perc_lat) + n_delay;
-                n_b = nb > INT_MAX ? INT_MAX : (int32_t)nb;
-            }
+        double gap_meas, closing;
+        if (M.lead_moving) {  // gap and closing speed to the moving lead
+            const double t = from_int(n) * q.dt;
+            gap_meas = ((d0 + lead_pos(M, t)) - x) + noise;
+            closing = v - lead_speed(M, t);
+        } else {
+            gap_meas = q.add(q.sub(d0, x), noise);
+            closing = v;
         }
+        bool reading = true;
+        if (M.perc) {  // the reading of step n + L describes step n
+            uint32_t h[4];
+            perc_halves(row, (uint64_t)((long long)n + M.perc_lat), M.perc_seed, h);
+            const double s32 = 1.0 / 4294967296.0;  // 2^-32
+            const double u1 = (double)h[0] * s32, u2 = (double)h[1] * s32;
+            const double u3 = (double)h[2] * s32, u4 = (double)h[3] * s32;
+            if (u4 < M.perc_drop) reading = false;
+            else gap_meas = gap_meas + M.perc_sigma * (2.0 * (((u1 + u2) + u3) - 1.5));
+        }
+        if (reading && gap_meas <= thr * closing) {
+            trig = true;
+            long long nb = ((long long)n + M.perc_lat) + n_delay;
+            n_b = nb > INT_MAX ? INT_MAX : (int32_t)nb;
+        }
+    }
+
+    // One RK4 step (all lanes of the warp together); true if the lane's rollout
+    // ended (stored).
+    __device__ __forceinline__ bool step(const ModelDev &M, const Ops &q, const OutDev &O,
+                                         uint64_t i)
+    {
+        const double dt = q.dt, h2 = q.h2, h6 = q.h6;
+        if (TTC && active && !trig) test_trigger(M, q);
         const double u = (trig && n >= n_b) ? M.a_cmd : 0.0;
 
         double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
         if (lagged) {
             a1 = a;
-            ka1 = (u - a1) * it;
-            a2 = a + h2 * ka1;
-            ka2 = (u - a2) * it;
-            a3 = a + h2 * ka2;
-            ka3 = (u - a3) * it;
-            a4 = a + dt * ka3;
-            ka4 = (u - a4) * it;
+            ka1 = q.mul(q.sub(u, a1), it);
+            a2 = q.add(a, q.mul(h2, ka1));
+            ka2 = q.mul(q.sub(u, a2), it);
+            a3 = q.add(a, q.mul(h2, ka2));
+            ka3 = q.mul(q.sub(u, a3), it);
+            a4 = q.add(a, q.mul(dt, ka3));
+            ka4 = q.mul(q.sub(u, a4), it);
         } else {
             a1 = a2 = a3 = a4 = u;
         }
@@ -274,33 +331,36 @@ struct Lane64 {
         // the stage actuator values are finite, so order keys compare them.)
         const bool dec = M.a_cmd <= 0.0;
         const long long kfirst = -okey(dec ? a1 : a4), klast = -okey(dec ? a4 : a1);
-        const bool pw = piece >= 0 && kfirst >= klo && klast <= khi;
-        const bool lines = __any_sync(__activemask(), pw && (piece == 1 || piece == 2));
-        double kv1, kv2, kv3, kv4, v2, v3, v4;
+        const bool pw = piece >= 0 && kfirst >= klo && klast <= khi && tame_speed(v);
+        const bool lines = __any_sync(kFull, active && pw && (piece == 1 || piece == 2));
+        double v2, v3, v4, xn, vn, an;
         if (pw) {
-            kv1 = accel_piece(v, a1, lines);
+            const double kv1 = accel_piece(q, v, a1, lines);
+            v2 = q.add(v, q.mul(h2, kv1));
+            const double kv2 = accel_piece(q, v2, a2, lines);
+            v3 = q.add(v, q.mul(h2, kv2));
+            const double kv3 = accel_piece(q, v3, a3, lines);
+            v4 = q.add(v, q.mul(dt, kv3));
+            const double kv4 = accel_piece(q, v4, a4, lines);
+            xn = q.combine(x, v, v2, v3, v4);
+            vn = q.combine(v, kv1, kv2, kv3, kv4);
+            an = lagged ? q.combine(a, ka1, ka2, ka3, ka4) : u;
+        } else if (active) {
+            const double kv1 = accel(v, a1);
             v2 = v + h2 * kv1;
-            kv2 = accel_piece(v2, a2, lines);
+            const double kv2 = accel(v2, a2);
             v3 = v + h2 * kv2;
-            kv3 = accel_piece(v3, a3, lines);
+            const double kv3 = accel(v3, a3);
             v4 = v + dt * kv3;
-            kv4 = accel_piece(v4, a4, lines);
-        } else {
-            kv1 = accel(v, a1);
-            v2 = v + h2 * kv1;
-            kv2 = accel(v2, a2);
-            v3 = v + h2 * kv2;
-            kv3 = accel(v3, a3);
-            v4 = v + dt * kv3;
-            kv4 = accel(v4, a4);
+            const double kv4 = accel(v4, a4);
+            xn = x + h6 * (((v + 2.0 * v2) + 2.0 * v3) + v4);
+            vn = v + h6 * (((kv1 + 2.0 * kv2) + 2.0 * kv3) + kv4);
+            an = lagged ? a + h6 * (((ka1 + 2.0 * ka2) + 2.0 * ka3) + ka4) : u;
         }
-
-        const double xn = x + h6 * (((v + 2.0 * v2) + 2.0 * v3) + v4);
-        const double vn = v + h6 * (((kv1 + 2.0 * kv2) + 2.0 * kv3) + kv4);
-        const double an = lagged ? a + h6 * (((ka1 + 2.0 * ka2) + 2.0 * ka3) + ka4) : u;
+        if (!active) return false;
 
         if (LEAD && M.lead_moving) {
-            const double t0 = (double)n * dt, t1 = (double)(n + 1) * dt;
+            const double t0 = from_int(n) * dt, t1 = from_int(n + 1) * dt;
             const double g1 = (d0 + lead_pos(M, t1)) - xn;
             if (g1 <= 0.0) {
                 const double g0 = (d0 + lead_pos(M, t0)) - x;
@@ -343,7 +403,48 @@ template <int CAP, bool LEAD, bool TTC>
 __global__ void __launch_bounds__(128, AEB_FP64_MIN_BLOCKS)
 k_rollout_fp64(ModelDev M, ParamsDev P, OutDev O, WorkDev W)
 {
-    rollout_driver<Lane64<CAP, LEAD, TTC>>(M, NoExtra{}, P, O, W, W.tile);
+    // Each lane owns one rollout at a time (Sec. V-A, one thread per sample); a
+    // lane whose rollout ends takes the next sample of its warp's ticket, so a
+    // warp keeps its lanes busy until the tickets run out instead of idling
+    // until its slowest rollout ends.  There is no wait on other warps or on
+    // the host: the loop ends when no lane holds a rollout.
+    __shared__ double cst[6][128];
+    cst[0][threadIdx.x] = 1.0;
+    cst[1][threadIdx.x] = 2.0;
+    cst[2][threadIdx.x] = -0.0;
+    cst[3][threadIdx.x] = M.dt;
+    cst[4][threadIdx.x] = M.h2;
+    cst[5][threadIdx.x] = M.h6;
+    __syncthreads();  // (read back per lane: register operands, see above)
+    const unsigned t = threadIdx.x ^ (unsigned)(W.n >> 63);
+    const Ops q{cst[0][t], cst[1][t], cst[2][t], cst[3][t], cst[4][t], cst[5][t]};
+    const unsigned lane = threadIdx.x & 31u;
+    WarpQueue wq;
+    Lane64<CAP, LEAD, TTC> L;
+    L.active = false;
+    L.x = L.v = L.a = L.d0 = L.gs = L.noise = L.k = L.it = L.thr = 0.0;
+    L.mg = L.f0 = L.f1 = L.r0 = L.r1 = L.cap = L.pa = L.pb = 0.0;
+    L.klo = L.khi = 0;
+    L.row = 0;
+    L.n = L.n_b = L.n_delay = 0;
+    L.piece = -1;
+    L.trig = L.lagged = L.ordered = false;
+    uint64_t pidx = 0, oidx = 0, kidx = 0;
+    double thr = M.ttc_thr;
+    unsigned need = kFull;
+    for (;;) {
+        while (need) {
+            const bool got = wq.take(need, W, W.tile, M.ttc_thr, pidx, oidx, kidx, thr);
+            bool ended = false;
+            if ((need >> lane) & 1u) {
+                L.active = got;
+                if (got) ended = L.init(M, P, O, pidx, oidx, kidx, thr);
+            }
+            need = __ballot_sync(kFull, ended);
+        }
+        if (!__any_sync(kFull, L.active)) return;
+        need = __ballot_sync(kFull, L.step(M, q, O, oidx));
+    }
 }
 
 template <int CAP, bool LEAD, bool TTC>

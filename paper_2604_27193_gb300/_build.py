@@ -26,6 +26,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = {
     "rollout_fp64.cu": ["-fmad=false"],
     "rollout_fp32.cu": ["-fmad=false"],
+    "order.cu": [],
     "reduce.cu": [],
     "reduce_noalloc.cu": [],
     "reduce_weighted.cu": [],

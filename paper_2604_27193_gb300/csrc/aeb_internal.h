@@ -55,17 +55,21 @@ struct TileDesc {
 };
 
 // Work split, handed to warps through one 64-bit counter that must be zero at
-// launch.  Flat mode (tiles == nullptr): samples [0, n) of one job in tiles of
-// `tile` samples, parameters and outputs at the same row, the model's TTC
-// threshold.  Table mode: tile t is tiles[t] of job jobs[tiles[t].job].
+// launch.  A launch walks positions: flat mode (tiles == nullptr), position p
+// is row row0 + p of the columns, with the model's TTC threshold; table mode,
+// position p is sample p % tile of tiles[p / tile] (a tile that holds fewer
+// samples leaves positions unused).  A warp's ticket is `tile` consecutive
+// positions, or, with a processing order, `tile` consecutive entries of perm.
 struct WorkDev {
-    uint64_t n;
+    uint64_t n;         // samples (fewer than 2^32 positions per launch)
     uint32_t tile;
     unsigned long long *counter;
     const TileDesc *tiles;
     uint64_t n_tiles;
     const JobDev *jobs;
-    uint64_t key_base;  // flat launches: perception-key row of sample 0
+    uint64_t key_base;  // flat launches: perception-key row of row 0
+    uint64_t row0;
+    const uint32_t *perm;  // the n positions in processing order (nullptr: natural order)
 };
 
 struct LaunchCfg {
@@ -87,11 +91,24 @@ inline uint32_t ticket_tile(const LaunchCfg &c)
     return (uint32_t)(c.tile_set ? c.tile : kTicketSamples);
 }
 
-// Launchers (asynchronous on `stream`; return a cudaError_t of the launch).
+// Launchers of one kernel (asynchronous on `stream`; return a cudaError_t of
+// the launch).
 cudaError_t launch_rollout_fp64(const ModelDev &m, const ParamsDev &p, const OutDev &o,
                                 const WorkDev &w, const LaunchCfg &cfg, cudaStream_t stream);
 cudaError_t launch_rollout_fp32(const ModelDev &m, const ParamsDev &p, const OutDev &o,
                                 const WorkDev &w, const LaunchCfg &cfg, cudaStream_t stream);
+
+// A whole rollout (order.cu): chooses the processing order, clears the ticket
+// counter and launches, in pieces if the work has more positions than one
+// launch takes.  `w` describes all of it (w.counter and w.perm are set here);
+// host_tiles is the host copy of w.tiles.  `scratch` holds rollout_scratch_bytes
+// of the work's positions, or only kCounterBytes: then the order is natural.
+constexpr size_t kCounterBytes = 256;
+size_t rollout_scratch_bytes(uint64_t positions, const ModelDev &m, aeb_precision precision);
+cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision precision,
+                           const OutDev &o, const WorkDev &w, const TileDesc *host_tiles,
+                           const LaunchCfg &cfg, void *scratch, size_t scratch_bytes,
+                           cudaStream_t stream);
 
 // Reduction: partial sums per block in fixed order, then one block finishes.
 struct RedPartial {

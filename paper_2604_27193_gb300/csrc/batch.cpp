@@ -98,24 +98,28 @@ extern "C" aeb_status aeb_batch_create(const aeb_model *model, const aeb_job *jo
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
-    const size_t o_counter = 0;
-    const size_t o_jobs = a256(sizeof(unsigned long long));
+    const size_t o_jobs = 0;
     const size_t o_tiles = o_jobs + a256(sizeof(JobDev) * n_jobs);
     const size_t o_red = o_tiles + a256(sizeof(TileDesc) * tiles.size());
     const size_t o_first = o_red + a256(sizeof(TileDesc) * red.size());
     const size_t o_part = o_first + a256(sizeof(uint32_t) * first.size());
-    const size_t bytes = o_part + a256(sizeof(RedPartial) * (red.size() + 1));
+    const size_t o_scratch = o_part + a256(sizeof(RedPartial) * (red.size() + 1));
+    size_t scratch = rollout_scratch_bytes((uint64_t)tiles.size() * T, md, precision);
 
     aeb_batch *b = new aeb_batch;
     b->device = dev;
     b->n_jobs = n_jobs;
-    e = cudaMalloc(&b->mem, bytes);
+    e = cudaMalloc(&b->mem, o_scratch + scratch);
+    if (e == cudaErrorMemoryAllocation && scratch > kCounterBytes) {
+        cudaGetLastError();
+        scratch = kCounterBytes;  // no room for a processing order: natural order
+        e = cudaMalloc(&b->mem, o_scratch + scratch);
+    }
     if (e != cudaSuccess) {
         delete b;
         return cuda_fail(e, "cudaMalloc(batch plan)");
     }
     char *base = static_cast<char *>(b->mem);
-    auto *counter = reinterpret_cast<unsigned long long *>(base + o_counter);
     auto *djobs = reinterpret_cast<JobDev *>(base + o_jobs);
     auto *dtiles = reinterpret_cast<TileDesc *>(base + o_tiles);
     auto *dred = reinterpret_cast<TileDesc *>(base + o_red);
@@ -147,11 +151,11 @@ extern "C" aeb_status aeb_batch_create(const aeb_model *model, const aeb_job *jo
     const OutDev od = out_dev(out);
     e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t le = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), cs);
-        if (le == cudaSuccess && !tiles.empty()) {
-            WorkDev w{total, T, counter, dtiles, (uint64_t)tiles.size(), djobs, 0};
-            le = (precision == AEB_FP64_PLAIN) ? launch_rollout_fp64(md, pd, od, w, cfg, cs)
-                                               : launch_rollout_fp32(md, pd, od, w, cfg, cs);
+        cudaError_t le = cudaSuccess;
+        if (!tiles.empty()) {
+            const WorkDev w{total, T, nullptr, dtiles, (uint64_t)tiles.size(), djobs, 0, 0, nullptr};
+            le = launch_rollout(md, pd, precision, od, w, tiles.data(), cfg, base + o_scratch,
+                                scratch, cs);
         }
         if (le == cudaSuccess)
             le = launch_reduce_jobs(out->status, out->x_ref, out->v_imp, out->n_steps, dred,

@@ -170,7 +170,6 @@ struct Region {
 std::mutex g_mu;
 std::map<std::pair<int, uintptr_t>, Region> g_scratch;
 
-constexpr size_t kCounterBytes = 256;
 size_t partial_bytes() { return sizeof(RedPartial) * 1024; }
 
 aeb_status scratch_for(cudaStream_t s, size_t bytes, void **out)
@@ -196,6 +195,52 @@ aeb_status scratch_for(cudaStream_t s, size_t bytes, void **out)
     return AEB_OK;
 }
 
+// Scratch of a rollout's processing order (6 B per sample, 100 MB at most),
+// from a pool of the library's own per device: allocated and freed in stream
+// order, so calls on any streams and threads share it safely, and no more than
+// kPoolKeep bytes stay allocated once the work is done.
+constexpr uint64_t kPoolKeep = uint64_t(256) << 20;
+std::map<int, cudaMemPool_t> g_pools;
+
+// nullptr if the memory cannot be had (or must not be allocated: a stream being
+// captured); the rollout then runs in natural order.
+void *order_alloc(size_t bytes, cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    int dev = 0;
+    void *p = nullptr;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+        cudaGetDevice(&dev) == cudaSuccess) {
+        cudaMemPool_t pool = nullptr;
+        {
+            std::lock_guard<std::mutex> lk(g_mu);
+            auto it = g_pools.find(dev);
+            if (it == g_pools.end()) {
+                cudaMemPoolProps props{};
+                props.allocType = cudaMemAllocationTypePinned;
+                props.location.type = cudaMemLocationTypeDevice;
+                props.location.id = dev;
+                uint64_t keep = kPoolKeep;
+                if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) pool = nullptr;
+                // (no reuse that would make one stream wait for another)
+                int off = 0;
+                if (pool &&
+                    (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+                     cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off) !=
+                         cudaSuccess)) {
+                    cudaMemPoolDestroy(pool);
+                    pool = nullptr;
+                }
+                it = g_pools.emplace(dev, pool).first;
+            }
+            pool = it->second;
+        }
+        if (pool && cudaMallocFromPoolAsync(&p, bytes, pool, s) == cudaSuccess) return p;
+    }
+    cudaGetLastError();  // not an error of the call
+    return nullptr;
+}
+
 std::mutex g_cfg_mu;
 LaunchCfg g_cfg[2] = {{128, 0, 256, false}, {128, 0, 32, false}};
 
@@ -206,13 +251,16 @@ aeb_status rollout_impl(const ModelDev &md, const ParamsDev &pd, uint64_t n,
     void *scratch = nullptr;
     aeb_status st = scratch_for(s, kCounterBytes + partial_bytes(), &scratch);
     if (st != AEB_OK) return st;
-    auto *counter = static_cast<unsigned long long *>(scratch);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(counter)");
     const LaunchCfg cfg = launch_cfg(precision);
-    WorkDev w{n, ticket_tile(cfg), counter, nullptr, 0, nullptr, key_base};
-    e = (precision == AEB_FP64_PLAIN) ? launch_rollout_fp64(md, pd, od, w, cfg, s)
-                                      : launch_rollout_fp32(md, pd, od, w, cfg, s);
+    const size_t want = rollout_scratch_bytes(n, md, precision);
+    void *order = want > kCounterBytes ? order_alloc(want, s) : nullptr;
+    const WorkDev w{n, ticket_tile(cfg), nullptr, nullptr, 0, nullptr, key_base, 0, nullptr};
+    cudaError_t e = launch_rollout(md, pd, precision, od, w, nullptr, cfg, order ? order : scratch,
+                                   order ? want : kCounterBytes, s);
+    if (order) {
+        const cudaError_t f = cudaFreeAsync(order, s);
+        if (e == cudaSuccess) e = f;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "rollout launch");
     return AEB_OK;
 }

@@ -1,0 +1,333 @@
+// order.cu -- the order in which a rollout launch takes its samples.
+//
+// A warp's 32 rollouts advance in lock step, so a warp is only as fast as its
+// lanes are alike: rollouts last 1.5 to 10 s, a launch of one generation lasts
+// as long as every warp's slowest lane, and in a long launch the lanes reach
+// their events (onset, breakpoints of r(D), the end) in different passes.
+// Taking the samples by predicted length, longest first, gives every warp
+// rollouts that start, turn and end together and leaves short ones for the
+// tail.  Results do not depend on the order: a sample's arithmetic never
+// depends on the lanes it shares a warp with.
+//
+// The prediction is a closed form in binary32 (coasting, then the braking that
+// the caps allow at full command, delayed by the area the actuator's ramp
+// loses, drag at a mean speed), 9 ms off the true length in the mean on the
+// single-scenario workload; it decides nothing but the order.  Samples whose
+// braking ends on the constant cap (saturated friction) come first: they last
+// longest, and a warp of them alone needs no actuator once it is there.
+//
+// Two kernels before the rollouts: bin every position by (cap class, length),
+// then scatter the positions to their bins' ranges (a counting sort; the
+// order inside a bin is free).  72 B read and 8 B written and read per
+// sample.
+#include <algorithm>
+#include <cmath>
+
+#include "rollout_common.cuh"
+
+namespace aeb {
+namespace {
+
+constexpr int kLenBins = 512;                 // over [0, horizon]
+constexpr int kClasses = 3;                   // constant cap, axle line, uncapped demand
+constexpr int kBins = kClasses * kLenBins;
+constexpr uint16_t kNoSample = 0xffff;        // a position no tile uses
+constexpr int kOrderThreads = 256;
+constexpr int kScatterItems = 16;             // positions per thread of the scatter
+// Positions ordered at a time, and so the bound on the scratch (100 MB).  A
+// longer launch runs in pieces; each piece's tail costs ~0.3 ms of ~40.
+constexpr uint64_t kOrderMax = uint64_t(1) << 24;
+constexpr uint64_t kNaturalMax = uint64_t(1) << 31;
+
+// Binary32 copies of the model's constants.
+struct OrderModel {
+    float D, g, rho_a2, hl, beta, phi_f, thr, lat, t_max, lv0, lb, lts, lxs;
+    int lumped, ttc, lead, moving;
+};
+
+struct Motion {  // coasting at -a0 until tb, then braking at -b
+    float v0, a0, tb, v1, x1, b;
+    __device__ float x(float t) const
+    {
+        if (t <= tb) return t * (v0 - 0.5f * a0 * t);
+        const float s = t - tb;
+        return x1 + s * (v1 - 0.5f * b * s);
+    }
+};
+
+// Predicted seconds until the rollout ends, and its cap class.
+__device__ __forceinline__ float predict(const OrderModel &M, const ParamsDev &P, const Row &row,
+                                         int &cls)
+{
+    auto f = [&](int j) { return (float)__ldg(P.col[j] + row.p); };
+    const float v0 = f(kV0), mu = f(kMu), gs = f(kGs), tau = f(kTau);
+    const float mh = mu * M.hl;
+    float r = M.D;
+    cls = 2;
+    if (M.lumped) {
+        const float c = __fdividef(mu * M.g, 1.0f + mh);
+        if (c < r) {
+            r = c;
+            cls = 0;
+        }
+    } else {
+        const float mg = mu * M.g;
+        const float im = __fdividef(1.0f, 1.0f - mh), ip = __fdividef(1.0f, 1.0f + mh);
+        const float lf = (mg * M.phi_f + (1.0f - M.beta) * M.D) * im;
+        const float lr = (mg * (1.0f - M.phi_f) + M.beta * M.D) * ip;
+        const float line = fminf(lf, lr);
+        if (line < r) {
+            r = line;
+            cls = 1;
+        }
+        if (mg <= r) {
+            r = mg;
+            cls = 0;
+        }
+    }
+    r = fmaxf(r, 1e-3f);
+    const float k = __fdividef(M.rho_a2 * f(kCd), f(kMass));
+    const float a0 = gs + k * v0 * v0;
+    // the ramp min(r, D (1 - exp(-t / tau))) as a step to r, delayed by the
+    // area it loses
+    const float w = fminf(fmaxf(1.0f - __fdividef(r, M.D), 1e-6f), 1.0f);
+    const float te = tau * fmaxf(1.0f + __fdividef(M.D - r, r) * __logf(w), 0.0f);
+    float td = f(kTdelay) + M.lat;
+    const float d0 = M.lead ? f(kD0) : 0.0f;
+    if (M.ttc) {  // coasting until the measured gap reaches thr times the closing speed
+        const float lb = M.moving ? M.lb : 0.0f;
+        const float c0 = v0 - M.lv0, C = f(kD0) + f(kNoise) - (float)row.thr * c0;
+        if (C > 0.0f) {
+            const float A = 0.5f * (lb - a0), B = c0 + (float)row.thr * (lb - a0);
+            const float q = B * B + 4.0f * A * C;
+            const float t = (q > 0.0f) ? __fdividef(2.0f * C, B + sqrtf(q)) : M.t_max;
+            td += (t > 0.0f) ? fminf(t, M.t_max) : M.t_max;
+        }
+    }
+    Motion m;
+    m.v0 = v0;
+    m.a0 = a0;
+    m.tb = td + te;
+    m.v1 = fmaxf(v0 - a0 * m.tb, 0.1f);
+    m.x1 = m.tb * (v0 - 0.5f * a0 * m.tb);
+    const float kv = k * m.v1 * m.v1, b = fmaxf(r + gs, 0.05f);
+    const float ts = m.tb + __fdividef(m.v1, b + kv * (1.0f / 3.0f));
+    m.b = b + 0.5f * kv;
+    const float sb = __fdividef(m.v1 * m.v1, 2.0f * m.b);  // braking distance
+    if (!M.lead) return ts;
+    if (!M.moving) {
+        const float d = d0 - m.x1;
+        if (d < 0.0f) return __fdividef(d0, v0);
+        if (sb < d) return ts;
+        // drag over the part of the braking distance that is driven
+        const float bc = b + kv * (1.0f - 0.5f * __fdividef(d, sb));
+        return m.tb + __fdividef(2.0f * d, m.v1 + sqrtf(fmaxf(m.v1 * m.v1 - 2.0f * bc * d, 0.0f)));
+    }
+    // moving lead: the first sign change of the gap over twelve parts of the
+    // time to stop
+    const float te12 = fminf(ts, M.t_max) * (1.0f / 12.0f);
+    float g0 = d0;
+    for (int i = 1; i <= 12; ++i) {
+        const float t = te12 * (float)i;
+        const float xl = (M.lb > 0.0f && t >= M.lts) ? M.lxs : t * (M.lv0 - 0.5f * M.lb * t);
+        const float g1 = d0 + xl - m.x(t);
+        if (g1 <= 0.0f) return t - te12 * (1.0f - __fdividef(g0, g0 - g1));
+        g0 = g1;
+    }
+    return ts;
+}
+
+// Pass 1: each position's bin and the bins' counts.
+__global__ void __launch_bounds__(kOrderThreads)
+k_order_keys(OrderModel M, ParamsDev P, WorkDev W, uint32_t positions,
+             uint32_t *__restrict__ hist, uint16_t *__restrict__ keys)
+{
+    __shared__ uint32_t sh[kBins];
+    for (int j = threadIdx.x; j < kBins; j += kOrderThreads) sh[j] = 0u;
+    __syncthreads();
+    const uint32_t step = gridDim.x * kOrderThreads;
+    for (uint32_t p = blockIdx.x * kOrderThreads + threadIdx.x; p < positions; p += step) {
+        uint16_t key = kNoSample;
+        if (!W.tiles || p % W.tile < W.tiles[p / W.tile].count) {
+            int cls;
+            const float t = predict(M, P, row_of(W, p, (double)M.thr), cls);
+            // longest first; a NaN counts as no time at all
+            int len = (t > 0.0f) ? (int)(fminf(t * __fdividef((float)kLenBins, M.t_max), 1e6f)) : 0;
+            len = len < kLenBins ? len : kLenBins - 1;
+            key = (uint16_t)(cls * kLenBins + (kLenBins - 1 - len));
+            atomicAdd(&sh[key], 1u);
+        }
+        keys[p] = key;
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < kBins; j += kOrderThreads)
+        if (sh[j]) atomicAdd(&hist[j], sh[j]);
+}
+
+// Pass 2: positions to their bins' ranges.  Each block ranks its positions in
+// shared memory and reserves one range per bin it holds.
+__global__ void __launch_bounds__(kOrderThreads)
+k_order_scatter(uint32_t positions, const uint32_t *__restrict__ hist,
+                uint32_t *__restrict__ cursor, const uint16_t *__restrict__ keys,
+                uint32_t *__restrict__ perm)
+{
+    constexpr int kPer = kBins / kOrderThreads;
+    static_assert(kBins % kOrderThreads == 0, "whole bins per thread");
+    __shared__ uint32_t cnt[kBins], base[kBins];
+    __shared__ uint32_t part[kOrderThreads / 32];
+    const int t = threadIdx.x;
+    // exclusive scan of the bin counts
+    uint32_t own[kPer], sum = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        own[j] = __ldg(hist + t * kPer + j);
+        sum += own[j];
+        cnt[t * kPer + j] = 0u;
+    }
+    uint32_t inc = sum;
+    for (int m = 1; m < 32; m <<= 1) {
+        const uint32_t o = __shfl_up_sync(kFull, inc, m);
+        if ((t & 31) >= m) inc += o;
+    }
+    if ((t & 31) == 31) part[t >> 5] = inc;
+    __syncthreads();
+    uint32_t run = inc - sum;
+    for (int w = 0; w < (t >> 5); ++w) run += part[w];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        base[t * kPer + j] = run;
+        run += own[j];
+    }
+    const uint32_t p0 = blockIdx.x * (uint32_t)(kOrderThreads * kScatterItems) + t;
+    uint32_t rank[kScatterItems];
+    uint16_t key[kScatterItems];
+#pragma unroll
+    for (int i = 0; i < kScatterItems; ++i) {
+        const uint32_t p = p0 + (uint32_t)i * kOrderThreads;
+        key[i] = p < positions ? keys[p] : kNoSample;
+        rank[i] = key[i] != kNoSample ? atomicAdd(&cnt[key[i]], 1u) : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int b = t + j * kOrderThreads;
+        if (cnt[b]) base[b] += atomicAdd(&cursor[b], cnt[b]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kScatterItems; ++i)
+        if (key[i] != kNoSample) perm[base[key[i]] + rank[i]] = p0 + (uint32_t)i * kOrderThreads;
+}
+
+OrderModel order_model(const ModelDev &m)
+{
+    OrderModel o;
+    o.D = std::max((float)-m.a_cmd, 1e-3f);
+    o.g = (float)m.g;
+    o.rho_a2 = (float)(0.5 * m.rho * m.area);
+    o.hl = (float)m.hl;
+    o.beta = (float)m.beta;
+    o.phi_f = (float)m.phi_f;
+    o.thr = (float)m.ttc_thr;
+    o.lat = (float)(m.perc_lat * m.dt);
+    o.t_max = (float)(m.n_max * m.dt);
+    o.lv0 = m.lead_moving ? (float)m.lead_v0 : 0.0f;
+    o.lb = (float)m.lead_decel;
+    o.lts = (float)m.lead_ts;
+    o.lxs = (float)m.lead_xs;
+    o.lumped = m.cap_mode == AEB_CAP_LUMPED;
+    o.ttc = m.trigger == AEB_TRIGGER_TTC;
+    o.lead = m.lead;
+    o.moving = m.lead_moving;
+    return o;
+}
+
+size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
+
+// Scratch of an ordered launch: the ticket counter, the bins' counts and
+// cursors (one clear covers the three), the keys and the order.
+struct Layout {
+    size_t hist = kCounterBytes, cursor = hist + a256(4 * kBins),
+           keys = cursor + a256(4 * kBins), perm, bytes;
+    explicit Layout(uint64_t positions)
+    {
+        perm = keys + a256(2 * positions);
+        bytes = perm + a256(4 * positions);
+    }
+};
+
+// Whether a launch of this many positions is worth ordering.  With at most
+// one warp per sub-partition (152 x 4 x 32 = 19,456 rollouts) a binary32 launch
+// lasts as long as its longest rollout in any order, and the two kernels would
+// add ~10 us to ~200.
+bool wants_order(uint64_t positions)
+{
+    return positions > 19456;
+}
+
+}  // namespace
+
+size_t rollout_scratch_bytes(uint64_t positions, const ModelDev &, aeb_precision)
+{
+    if (!wants_order(positions)) return kCounterBytes;
+    return Layout(std::min(positions, kOrderMax)).bytes;
+}
+
+cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision precision,
+                           const OutDev &o, const WorkDev &w, const TileDesc *host_tiles,
+                           const LaunchCfg &cfg, void *scratch, size_t scratch_bytes,
+                           cudaStream_t s)
+{
+    const uint64_t all = w.tiles ? w.n_tiles * w.tile : w.n;
+    const bool order = m.n_max > 0 && wants_order(all) &&
+                       scratch_bytes >= rollout_scratch_bytes(all, m, precision);
+    const uint64_t piece = order ? kOrderMax : kNaturalMax;  // positions per launch
+    const uint64_t unit = w.tiles ? piece / w.tile : piece;   // tiles or rows per launch
+    const uint64_t total = w.tiles ? w.n_tiles : w.n;
+    char *base = static_cast<char *>(scratch);
+    const Layout lay(std::min(all, kOrderMax));
+    for (uint64_t first = 0; first < total; first += unit) {
+        const uint64_t len = std::min(unit, total - first);
+        WorkDev k = w;
+        k.counter = reinterpret_cast<unsigned long long *>(base);
+        k.perm = nullptr;
+        uint64_t positions = len;
+        if (w.tiles) {
+            k.tiles = w.tiles + first;
+            k.n_tiles = len;
+            positions = len * w.tile;
+            if (len < total) {
+                k.n = 0;
+                for (uint64_t t = first; t < first + len; ++t) k.n += host_tiles[t].count;
+            }
+        } else {
+            k.row0 = w.row0 + first;
+            k.n = len;
+        }
+        cudaError_t e = cudaMemsetAsync(base, 0, order ? lay.keys : sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+        if (order) {
+            auto *hist = reinterpret_cast<uint32_t *>(base + lay.hist);
+            auto *cursor = reinterpret_cast<uint32_t *>(base + lay.cursor);
+            auto *keys = reinterpret_cast<uint16_t *>(base + lay.keys);
+            auto *perm = reinterpret_cast<uint32_t *>(base + lay.perm);
+            const uint32_t np = (uint32_t)positions;
+            const uint32_t kb = std::min<uint32_t>((np + kOrderThreads - 1) / kOrderThreads, 152 * 8);
+            k_order_keys<<<kb, kOrderThreads, 0, s>>>(order_model(m), p, k, np, hist, keys);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            constexpr uint32_t kChunk = kOrderThreads * kScatterItems;
+            k_order_scatter<<<(np + kChunk - 1) / kChunk, kOrderThreads, 0, s>>>(np, hist, cursor,
+                                                                               keys, perm);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            k.perm = perm;
+        }
+        e = precision == AEB_FP64_PLAIN ? launch_rollout_fp64(m, p, o, k, cfg, s)
+                                        : launch_rollout_fp32(m, p, o, k, cfg, s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace aeb

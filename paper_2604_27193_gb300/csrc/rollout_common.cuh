@@ -8,7 +8,6 @@
 namespace aeb {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr uint64_t kNone = ~0ull;
 
 __device__ __forceinline__ unsigned lanemask_lt()
 {
@@ -17,73 +16,87 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
-// A claimed tile: `count` samples with parameters at rows p0.. and outputs at
-// rows o0.., and the TTC threshold of their job.  Warp-uniform.
-struct Tile {
-    uint64_t p0, o0, k0;  // parameter, output and perception-key rows of the first sample
-    int count;
+// The rows of a position: parameters, outputs, perception key, and the TTC
+// threshold of its job.
+struct Row {
+    uint64_t p, o, k;
     double thr;
-    bool ok;
 };
-
-// Claim the next tile (all 32 lanes call together; lane 0 takes the ticket).
-__device__ __forceinline__ Tile claim_tile(const WorkDev &w, uint32_t tile_size, double model_thr)
+__device__ __forceinline__ Row row_of(const WorkDev &w, uint32_t pos, double model_thr)
 {
-    unsigned long long t = 0;
-    if ((threadIdx.x & 31u) == 0) t = atomicAdd(w.counter, 1ull);
-    t = __shfl_sync(kFull, t, 0);
-    Tile r;
+    Row r;
     if (!w.tiles) {
-        const uint64_t start = (uint64_t)t * tile_size;
-        r.ok = start < w.n;
-        r.p0 = r.o0 = start;
-        r.k0 = w.key_base + start;
-        r.count = r.ok ? (int)((w.n - start < (uint64_t)tile_size) ? w.n - start : tile_size) : 0;
+        r.p = r.o = w.row0 + pos;
+        r.k = w.key_base + r.p;
         r.thr = model_thr;
     } else {
-        r.ok = t < w.n_tiles;
-        r.count = 0;
-        r.p0 = r.o0 = r.k0 = 0;
-        r.thr = model_thr;
-        if (r.ok) {
-            const TileDesc d = w.tiles[t];
-            const JobDev j = w.jobs[d.job];
-            r.p0 = j.param_offset + d.first;
-            r.o0 = j.out_offset + d.first;
-            r.k0 = j.key_offset + d.first;
-            r.count = (int)d.count;
-            r.thr = j.ttc_thr;
-        }
+        const uint32_t t = pos / w.tile;
+        const TileDesc d = w.tiles[t];
+        const JobDev j = w.jobs[d.job];
+        const uint64_t i = d.first + (pos - t * w.tile);
+        r.p = j.param_offset + i;
+        r.o = j.out_offset + i;
+        r.k = j.key_offset + i;
+        r.thr = j.ttc_thr;
     }
     return r;
 }
 
-// Number of tiles a launch walks.
-__host__ __forceinline__ uint64_t tiles_of(const WorkDev &w, uint32_t tile_size)
+// A claimed ticket: entries [start, start + count) of the processing order.
+// Warp-uniform.
+struct Ticket {
+    uint32_t start;
+    int count;
+    bool ok;
+};
+
+// Claim the next ticket (all 32 lanes call together; lane 0 takes it).
+__device__ __forceinline__ Ticket claim_ticket(const WorkDev &w)
 {
-    return w.tiles ? w.n_tiles : (w.n + tile_size - 1) / tile_size;
+    unsigned long long t = 0;
+    if ((threadIdx.x & 31u) == 0) t = atomicAdd(w.counter, 1ull);
+    t = __shfl_sync(kFull, t, 0);
+    Ticket r;
+    const uint64_t start = (uint64_t)t * w.tile;
+    r.start = (uint32_t)start;
+    if (w.tiles && !w.perm) {
+        r.ok = t < w.n_tiles;
+        r.count = r.ok ? (int)w.tiles[t].count : 0;
+    } else {
+        r.ok = start < w.n;
+        r.count = r.ok ? (int)((w.n - start < (uint64_t)w.tile) ? w.n - start : w.tile) : 0;
+    }
+    return r;
+}
+__device__ __forceinline__ uint32_t position(const WorkDev &w, uint32_t entry)
+{
+    return w.perm ? __ldg(w.perm + entry) : entry;
 }
 
-// A warp's cursor into the sample tiles.  All 32 lanes call take() together
-// with the same `need` mask (the lanes whose rollout just ended).  Each lane
-// in `need` receives the next unclaimed sample of the warp's tile (its
-// parameter row, output row and TTC threshold); when the tile is used up the
-// warp claims the next tile.  Lanes get false once every tile has been
-// claimed.  Per-sample results never depend on which warp runs a sample.
+// Number of tickets a launch hands out.
+__host__ __forceinline__ uint64_t tickets_of(const WorkDev &w)
+{
+    return (w.tiles && !w.perm) ? w.n_tiles : (w.n + w.tile - 1) / w.tile;
+}
+
+// A warp's cursor into its ticket.  All 32 lanes call take() together with the
+// same `need` mask (the lanes whose rollout just ended).  Each lane in `need`
+// receives the position of the next unclaimed sample of the warp's ticket;
+// when it is used up the warp claims the next.  Lanes get false once every
+// ticket has been claimed.  Per-sample results never depend on which warp runs
+// a sample.
 struct WarpQueue {
-    Tile cur{};
+    Ticket cur{0, 0, false};
     int used = 0;
     bool dry = false;
 
-    __device__ __forceinline__ bool take(unsigned need, const WorkDev &w, uint32_t tile_size,
-                                         double model_thr, uint64_t &pidx, uint64_t &oidx,
-                                         uint64_t &kidx, double &thr)
+    __device__ __forceinline__ bool take(unsigned need, const WorkDev &w, uint32_t &pos)
     {
         const unsigned lane = threadIdx.x & 31u;
         bool mine = false;
         while (need && !dry) {
             if (used >= cur.count) {
-                cur = claim_tile(w, tile_size, model_thr);
+                cur = claim_ticket(w);
                 used = 0;
                 if (!cur.ok) {
                     dry = true;
@@ -94,10 +107,7 @@ struct WarpQueue {
             const bool got = ((need >> lane) & 1u) && (int)rank < cur.count - used;
             if (got) {
                 mine = true;
-                pidx = cur.p0 + used + rank;
-                oidx = cur.o0 + used + rank;
-                kidx = cur.k0 + used + rank;
-                thr = cur.thr;
+                pos = position(w, cur.start + used + rank);
             }
             const unsigned taken = __ballot_sync(kFull, got);
             used += __popc(taken);

@@ -77,22 +77,24 @@ constexpr int kThreads = 32 * kWarps;
 
 // A prepared per-sample record in the warp's tile, sample-major: the fields
 // the lane that takes the sample loads into registers (R_*), then the block it
-// keeps in its shared-memory column (C_*, copied by the whole warp when lanes
-// refill).  Integer fields are stored as their bits.  The TTC fields exist only
-// in the TTC-trigger kernel; -s dt = 2 (-s dt/2) exactly, p4 = -np4, np1 = -1
+// keeps in its shared-memory column (the position and C_*, copied by the whole
+// warp when lanes refill).  Integer fields are stored as their bits.  The TTC
+// fields exist only in the TTC-trigger kernels, the key row only in those with
+// per-step perception; -s dt = 2 (-s dt/2) exactly, p4 = -np4, np1 = -1
 // when tau > 0 (else 0) and (1 - mP)^(K-1) are derived where needed.
-enum { R_W0H, R_W0L, R_G0H, R_G0L, R_NH2S, R_NH6S, R_NMP, R_KIND, R_C0 };
+enum { R_W0H, R_W0L, R_G0H, R_G0L, R_NH2S, R_NH6S, R_NMP, R_KIND, R_POS, R_C0 };
 enum {
     C_NDELAY, C_GS, C_S, C_SIGMA, C_F0, C_F1, C_R0, C_R1, C_MG, C_NP2, C_NP3, C_NP4,
     C_NBASE,                               // fields of every kernel
-    C_NZ = C_NBASE, C_THRH, C_THRL, C_NTTC  // TTC trigger only
+    C_NZ = C_NBASE, C_THRH, C_THRL, C_NTTC,  // TTC trigger only
+    C_KLO = C_NTTC, C_KHI, C_NPERC           // perception-key row (two words)
 };
-template <bool TTC>
-__host__ __device__ constexpr int copy_fields() { return TTC ? C_NTTC : C_NBASE; }
+template <bool TTC, bool PERC>
+__host__ __device__ constexpr int copy_fields() { return PERC ? C_NPERC : TTC ? C_NTTC : C_NBASE; }
 // Words per record: odd, so that 32 lanes reading one field of 32 records, or
 // one lane's record read by 32 lanes, hit 32 different banks.
-template <bool TTC>
-__host__ __device__ constexpr int rec_stride() { return (R_C0 + copy_fields<TTC>()) | 1; }
+template <bool TTC, bool PERC>
+__host__ __device__ constexpr int rec_stride() { return (R_C0 + copy_fields<TTC, PERC>()) | 1; }
 enum { K_RUN = 0, K_INVALID, K_CONTACT0, K_STOP0, K_HORIZON0 };
 
 // The lead vehicle, a template parameter of the kernel (so that a stationary
@@ -161,21 +163,27 @@ __device__ __forceinline__ int32_t steps_to_reach_f32(double t, double dt, float
     return (int32_t)n;
 }
 
-// Prepare samples [start, start + cnt) of a tile (TTC threshold thr) into the
-// warp's records (sample-major, rec_stride words each).  Kept out of line: it
+// Prepare the samples of a ticket (entries [start, start + cnt) of the
+// processing order) into the warp's records (sample-major, rec_stride words each).  Kept out of line: it
 // runs once per tile, and its binary64 code inlined into the kernel cost the
 // step loop ~3 % (measured on the single-scenario workload).
-template <int LEAD, bool TTC>
+template <int LEAD, bool TTC, bool PERC>
 __device__ __noinline__ void prep_tile(const ModelDev &M, const ModelF32 &F, const ParamsDev &P,
-                                          uint64_t start, int cnt, double thr, float *tf)
+                                       const WorkDev &W, uint32_t start, int cnt, float *tf)
 {
-    constexpr int RS = rec_stride<TTC>();
+    constexpr int RS = rec_stride<TTC, PERC>();
     for (int j = threadIdx.x & 31; j < cnt; j += 32) {
-        const uint64_t i = start + j;
+        const uint32_t pos = position(W, start + (uint32_t)j);
+        const Row rows = row_of(W, pos, M.ttc_thr);
         float *rc = tf + j * RS;
         float *cp = rc + R_C0;
+        rc[R_POS] = __int_as_float((int)pos);
+        if (PERC) {
+            cp[C_KLO] = __int_as_float((int)(uint32_t)rows.k);
+            cp[C_KHI] = __int_as_float((int)(uint32_t)(rows.k >> 32));
+        }
         double f[AEB_NFIELDS];
-        load_fields(P, i, f);
+        load_fields(P, rows.p, f);
         int kind = K_RUN, nd = 0;
         if (!sample_valid(f)) {
             kind = K_INVALID;
@@ -246,7 +254,7 @@ __device__ __noinline__ void prep_tile(const ModelDev &M, const ModelF32 &F, con
         }
         rc[R_NMP] = nmp;
         if (TTC) {  // (g + noise) - thr v scaled by sigma: G + sigma noise - (sigma thr / s) w
-            const double ts = thr * (sd * r6);  // sigma / s
+            const double ts = rows.thr * (sd * r6);  // sigma / s
             const float tsh = __double2float_rn(ts);
             cp[C_NZ] = __double2float_rn(sigma * f[kNoise]);
             cp[C_THRH] = tsh;
@@ -257,22 +265,24 @@ __device__ __noinline__ void prep_tile(const ModelDev &M, const ModelF32 &F, con
 
 // Per-lane values read only on rare paths (piece changes, slow steps, the TTC
 // test, records) live in a column of the warp's shared slab, to keep the step
-// loop's register budget small: the lane's own fields, its rows, then the
-// record block C_* (both written by the whole warp at refill).  Lane-major
+// loop's register budget small: the lane's own fields, its sample's position,
+// then the record block C_* (both written by the whole warp at refill).  Lane-major
 // with an odd stride, so that 32 lanes reading one field, or 32 lanes writing
 // one lane's column, hit 32 different banks.
 enum {
     L_U, L_ETHK, L_NB, L_NCHK, L_NP1, L_QF,                       // the lane's (NCHK: TTC)
-    L_PIDXLO, L_PIDXHI, L_IDXLO, L_IDXHI, L_KIDXLO, L_KIDXHI,     // rows (two words each)
+    L_POS,                                                        // the sample's position
     L_C0,                                                         // the record block
     L_NDELAY = L_C0 + C_NDELAY, L_GS = L_C0 + C_GS, L_S = L_C0 + C_S,
     L_SIGMA = L_C0 + C_SIGMA, L_F0 = L_C0 + C_F0, L_F1 = L_C0 + C_F1, L_R0 = L_C0 + C_R0,
     L_R1 = L_C0 + C_R1, L_MG = L_C0 + C_MG, L_NP2 = L_C0 + C_NP2, L_NP3 = L_C0 + C_NP3,
-    L_NP4 = L_C0 + C_NP4, L_NZ = L_C0 + C_NZ, L_THRH = L_C0 + C_THRH, L_THRL = L_C0 + C_THRL
+    L_NP4 = L_C0 + C_NP4, L_NZ = L_C0 + C_NZ, L_THRH = L_C0 + C_THRH, L_THRL = L_C0 + C_THRL,
+    L_KLO = L_C0 + C_KLO, L_KHI = L_C0 + C_KHI
 };
-template <bool TTC>
-__host__ __device__ constexpr int cold_stride() { return (L_C0 + copy_fields<TTC>()) | 1; }
-static_assert(L_C0 - L_PIDXLO + C_NTTC <= 32, "a column's rows and record block fit one warp");
+template <bool TTC, bool PERC>
+__host__ __device__ constexpr int cold_stride() { return (L_C0 + copy_fields<TTC, PERC>()) | 1; }
+static_assert(1 + C_NPERC <= 32, "a column's position and record block fit one warp");
+static_assert(R_C0 == R_POS + 1 && L_C0 == L_POS + 1, "the position precedes the record block");
 
 template <int LEAD, bool TTC, bool PERC>
 struct Lane32 {
@@ -291,11 +301,6 @@ struct Lane32 {
     __device__ __forceinline__ int ci(int f) const { return __float_as_int(cold[f]); }
     __device__ __forceinline__ void set_ci(int f, int x) { cold[f] = __int_as_float(x); }
     __device__ __forceinline__ float np1() const { return cf(L_NP1); }  // -p1
-    __device__ __forceinline__ uint64_t pidx() const
-    {
-        return (uint64_t)(uint32_t)ci(L_PIDXLO) | ((uint64_t)(uint32_t)ci(L_PIDXHI) << 32);
-    }
-
     // Select the line of r(D) that is the minimum at demand D (ties: the
     // flatter line, which stays the minimum to the right), its next breakpoint
     // B, and the threshold on e beyond which a step's largest demand
@@ -677,7 +682,7 @@ struct Lane32 {
 
     __device__ __forceinline__ uint64_t krow() const
     {
-        return (uint64_t)(uint32_t)ci(L_KIDXLO) | ((uint64_t)(uint32_t)ci(L_KIDXHI) << 32);
+        return (uint64_t)(uint32_t)ci(L_KLO) | ((uint64_t)(uint32_t)ci(L_KHI) << 32);
     }
 
     // The trigger fires at step k (its onset step n_b = k + L + n_delay); the
@@ -814,16 +819,18 @@ struct Lane32 {
         n = n0;
     }
 
-    // Take the prepared record rc (parameter row pi, output row i); true if
-    // the sample ended at once (stored).  The record block and the rows reach
-    // the lane's column from the whole warp afterwards (copy_records).
+    // Take the prepared record rc; true if the sample ended at once (stored).
+    // The record block and the position reach the lane's column from the whole
+    // warp afterwards (copy_records).
     __device__ __forceinline__ bool init(const ModelDev &M, const ParamsDev &P, const OutDev &O,
-                                         uint64_t pi, uint64_t i, const float *rc)
+                                         const WorkDev &W, const float *rc)
     {
         const int kind = __float_as_int(rc[R_KIND]);
         const int32_t n_delay = __float_as_int(rc[R_C0 + C_NDELAY]);
         if (kind != K_RUN) {
             const int32_t on = TTC ? -1 : n_delay;
+            const Row rows = row_of(W, (uint32_t)__float_as_int(rc[R_POS]), M.ttc_thr);
+            const uint64_t pi = rows.p, i = rows.o;
             if (kind == K_INVALID) {
                 const double nan = __longlong_as_double(0x7ff8000000000000ll);
                 store_out(O, i, AEB_INVALID, nan, nan, nan, nan, 0, -1);
@@ -868,30 +875,22 @@ struct Lane32 {
 };
 
 // After lanes took samples cursor, cursor + 1, ... of the tile (the lanes of
-// `taken`, in lane order): the rows and the record block of those in `keep`
+// `taken`, in lane order): the position and the record block of those in `keep`
 // reach their columns, written by the whole warp (lane t: word t of the
-// column's rows-and-record part; consecutive words, so no bank conflicts),
-// instead of ~20 loads and stores by each refilling lane alone.
-template <bool TTC>
-__device__ __forceinline__ void copy_records(float *coldw, const float *tf, const Tile &tile,
-                                             int cursor, unsigned taken, unsigned keep)
+// column's copied part; consecutive words, so no bank conflicts), instead of
+// ~20 loads and stores by each refilling lane alone.
+template <bool TTC, bool PERC>
+__device__ __forceinline__ void copy_records(float *coldw, const float *tf, int cursor,
+                                             unsigned taken, unsigned keep)
 {
-    constexpr int NC = copy_fields<TTC>(), CS = cold_stride<TTC>(), RS = rec_stride<TTC>();
+    constexpr int NC = 1 + copy_fields<TTC, PERC>(), CS = cold_stride<TTC, PERC>(),
+                  RS = rec_stride<TTC, PERC>();
     const int t = (int)(threadIdx.x & 31u);
-    const uint64_t base = t < 2 ? tile.p0 : t < 4 ? tile.o0 : tile.k0;  // rows (t < 6)
     int r = 0;
     for (unsigned tk = taken; tk; tk &= tk - 1, ++r) {
         const int l = __ffs(tk) - 1;
         if (!((keep >> l) & 1u)) continue;
-        const int slot = cursor + r;
-        float w = 0.0f;
-        if (t < L_C0 - L_PIDXLO) {
-            const uint64_t v = base + (uint64_t)slot;
-            w = __int_as_float((int)(uint32_t)((t & 1) ? (v >> 32) : v));
-        } else if (t < L_C0 - L_PIDXLO + NC) {
-            w = tf[slot * RS + R_C0 + (t - (L_C0 - L_PIDXLO))];
-        }
-        if (t < L_C0 - L_PIDXLO + NC) coldw[l * CS + L_PIDXLO + t] = w;
+        if (t < NC) coldw[l * CS + L_POS + t] = tf[(cursor + r) * RS + R_POS + t];
     }
     __syncwarp();  // the columns are read by their lanes from here on
 }
@@ -907,7 +906,7 @@ enum {
     B_C, B_S, B_SIGMA, B_NF
 };
 enum { B_G1H = B_A1, B_G1L = B_A2, B_W1H = B_A3, B_W1L = B_A4 };
-enum { B_IDXLO, B_IDXHI, B_PIDXLO, B_PIDXHI, B_STATUS, B_N, B_LEN, B_ONSET, B_NI };
+enum { B_POS, B_STATUS, B_N, B_LEN, B_ONSET, B_NI };
 constexpr int kBatchWords = (B_NF + B_NI) * 32;
 // Per-step perception: readings of up to kBandSlots lanes near their trigger,
 // kBandCache steps each, in the margin's units (+inf: missing), and per slot
@@ -922,7 +921,7 @@ constexpr int kBandState = 2 * AEB_FP32_WINDOW + 4;
 template <bool TTC, bool PERC>
 __host__ __device__ constexpr int warp_words(int T)
 {
-    return rec_stride<TTC>() * T + kBatchWords + cold_stride<TTC>() * 32 +
+    return rec_stride<TTC, PERC>() * T + kBatchWords + cold_stride<TTC, PERC>() * 32 +
            (PERC ? kBandSlots * (kBandCache + G_NI + kBandState) : 0);
 }
 template <bool TTC, bool PERC>
@@ -937,15 +936,13 @@ __host__ __device__ constexpr size_t smem_per_block(int T)
 template <int LEAD, bool TTC, bool PERC>
 __device__ __forceinline__ void flush_batch(const ModelDev &M, const ModelF32 &F,
                                             const ParamsDev &P, const OutDev &O,
-                                            const float *bf, const int *bi, int count)
+                                            const WorkDev &W, const float *bf, const int *bi, int count)
 {
     __syncwarp();
     const int j = threadIdx.x & 31;
     if (j < count) {
-        const uint64_t i = (uint64_t)(uint32_t)bi[B_IDXLO * 32 + j] |
-                           ((uint64_t)(uint32_t)bi[B_IDXHI * 32 + j] << 32);
-        const uint64_t pi = (uint64_t)(uint32_t)bi[B_PIDXLO * 32 + j] |
-                            ((uint64_t)(uint32_t)bi[B_PIDXHI * 32 + j] << 32);
+        const Row rows = row_of(W, (uint32_t)bi[B_POS * 32 + j], M.ttc_thr);
+        const uint64_t i = rows.o, pi = rows.p;
         const int len = bi[B_LEN * 32 + j] & 0xff;
         const int trel = (bi[B_LEN * 32 + j] >> 8) - 1;  // trigger step in the window (-1: none)
         int32_t on = bi[B_ONSET * 32 + j];
@@ -1051,10 +1048,10 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
     const unsigned lane = threadIdx.x & 31u;
     const int T = (int)W.tile;
     float *tf = smem + (threadIdx.x >> 5) * warp_words<TTC, PERC>(T);
-    float *bf = tf + rec_stride<TTC>() * T;
+    float *bf = tf + rec_stride<TTC, PERC>() * T;
     int *bi = reinterpret_cast<int *>(bf + B_NF * 32);
     float *coldw = bf + kBatchWords;
-    float *rdg = coldw + cold_stride<TTC>() * 32;  // band readings (per-step perception)
+    float *rdg = coldw + cold_stride<TTC, PERC>() * 32;  // band readings (per-step perception)
     int *btag = reinterpret_cast<int *>(rdg + kBandSlots * kBandCache);
     float *sst = reinterpret_cast<float *>(btag + kBandSlots * G_NI);  // band window states
     if (PERC && (int)lane < kBandSlots) btag[lane * G_NI + G_CNT] = 0;  // nothing cached
@@ -1068,11 +1065,11 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
         return rdg + sl * kBandCache + (n - btag[sl * G_NI + G_STEP]);
     };
 
-    Tile tile{};
+    Ticket tile{0, 0, false};
     int cursor = 0, bcount = 0;
     bool dry = false;
     Lane32<LEAD, TTC, PERC> L;
-    L.cold = coldw + lane * cold_stride<TTC>();
+    L.cold = coldw + lane * cold_stride<TTC, PERC>();
     bool active = false;
     unsigned need = kFull;
     for (;;) {
@@ -1083,7 +1080,7 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
                         if ((need >> lane) & 1u) active = false;
                         break;
                     }
-                    const Tile nt = claim_tile(W, (uint32_t)T, M.ttc_thr);
+                    const Ticket nt = claim_ticket(W);
                     if (!nt.ok) {
                         dry = true;
                         continue;
@@ -1091,7 +1088,7 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
                     tile = nt;
                     cursor = 0;
                     __syncwarp();  // every lane has read its record of the previous tile
-                    prep_tile<LEAD, TTC>(M, F, P, tile.p0, tile.count, tile.thr, tf);
+                    prep_tile<LEAD, TTC, PERC>(M, F, P, W, tile.start, tile.count, tf);
                     __syncwarp();
                 }
                 const unsigned rank = __popc(need & lanemask_lt());
@@ -1100,17 +1097,16 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
                 if (got) {
                     const int slot = cursor + (int)rank;
                     active = true;
-                    ended = L.init(M, P, O, tile.p0 + slot, tile.o0 + slot,
-                                   tf + slot * rec_stride<TTC>());
+                    ended = L.init(M, P, O, W, tf + slot * rec_stride<TTC, PERC>());
                 }
                 const unsigned taken = __ballot_sync(kFull, got);
                 const unsigned endm = __ballot_sync(kFull, ended);
-                copy_records<TTC>(coldw, tf, tile, cursor, taken, taken & ~endm);
+                copy_records<TTC, PERC>(coldw, tf, cursor, taken, taken & ~endm);
                 cursor += __popc(taken);
                 need = (need & ~taken) | endm;
             }
             if (!__any_sync(kFull, active)) {
-                flush_batch<LEAD, TTC, PERC>(M, F, P, O, bf, bi, bcount);
+                flush_batch<LEAD, TTC, PERC>(M, F, P, O, W, bf, bi, bcount);
                 return;
             }
         }
@@ -1151,7 +1147,7 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
             if (bm) {
                 const int rank = __popc(bm & lanemask_lt());
                 if (((bm >> lane) & 1u) && rank < kBandSlots) slot = rank;
-                const int klo = L.ci(L_KIDXLO), khi = L.ci(L_KIDXHI);
+                const int klo = L.ci(L_KLO), khi = L.ci(L_KHI);
                 bool miss = false;
                 if (slot >= 0) {
                     const int *tg = btag + slot * G_NI;
@@ -1295,7 +1291,7 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
         if (endm) {
             const int cnt = __popc(endm);
             if (bcount + cnt > 32) {
-                flush_batch<LEAD, TTC, PERC>(M, F, P, O, bf, bi, bcount);
+                flush_batch<LEAD, TTC, PERC>(M, F, P, O, W, bf, bi, bcount);
                 bcount = 0;
             }
             if (ended) {
@@ -1307,10 +1303,7 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
                 bf[B_NH6S * 32 + j] = L.nh6s;
                 bf[B_S * 32 + j] = L.cf(L_S);
                 bf[B_SIGMA * 32 + j] = L.cf(L_SIGMA);
-                bi[B_IDXLO * 32 + j] = L.ci(L_IDXLO);
-                bi[B_IDXHI * 32 + j] = L.ci(L_IDXHI);
-                bi[B_PIDXLO * 32 + j] = L.ci(L_PIDXLO);
-                bi[B_PIDXHI * 32 + j] = L.ci(L_PIDXHI);
+                bi[B_POS * 32 + j] = L.ci(L_POS);
                 bi[B_ONSET * 32 + j] = L.onset();
                 if (replay) {
                     bf[B_E * 32 + j] = L.e;
@@ -1391,14 +1384,11 @@ cudaError_t launch_t(const ModelDev &m, const ParamsDev &p, const OutDev &o, con
     if (e != cudaSuccess) return e;
     if (occ < 1) occ = 1;
     if (per_sm <= 0 || per_sm > occ) per_sm = occ;
-    WorkDev wt = w;
-    wt.tile = (uint32_t)T;
-    const uint64_t tiles = tiles_of(wt, (uint32_t)T);
     uint64_t blocks = (uint64_t)sms * per_sm;
-    const uint64_t need_blocks = (tiles + kWarps - 1) / kWarps;
+    const uint64_t need_blocks = (tickets_of(w) + kWarps - 1) / kWarps;
     if (need_blocks < blocks) blocks = need_blocks;
     if (blocks < 1) blocks = 1;
-    kern<<<(unsigned)blocks, kThreads, smem, s>>>(m, to_f32(m), p, o, wt);
+    kern<<<(unsigned)blocks, kThreads, smem, s>>>(m, to_f32(m), p, o, w);
     return cudaGetLastError();
 }
 

@@ -216,18 +216,18 @@ struct Lane64 {
     }
 
     __device__ __forceinline__ bool init(const ModelDev &M, const ParamsDev &P,
-                                         const OutDev &O, uint64_t pi, uint64_t i, uint64_t ki,
-                                         double thr_job)
+                                         const OutDev &O, const Row &rows)
     {
         double f[AEB_NFIELDS];
-        load_fields(P, pi, f);
-        thr = thr_job;
+        const uint64_t i = rows.o;
+        load_fields(P, rows.p, f);
+        thr = rows.thr;
         if (!sample_valid(f)) {
             const double nan = __longlong_as_double(0x7ff8000000000000ll);
             store_out(O, i, AEB_INVALID, nan, nan, nan, nan, 0, -1);
             return true;
         }
-        row = ki;
+        row = rows.k;
         d0 = f[kD0];
         gs = f[kGs];
         noise = f[kNoise];
@@ -429,16 +429,20 @@ k_rollout_fp64(ModelDev M, ParamsDev P, OutDev O, WorkDev W)
     L.n = L.n_b = L.n_delay = 0;
     L.piece = -1;
     L.trig = L.lagged = L.ordered = false;
-    uint64_t pidx = 0, oidx = 0, kidx = 0;
-    double thr = M.ttc_thr;
+    uint64_t oidx = 0;
     unsigned need = kFull;
     for (;;) {
         while (need) {
-            const bool got = wq.take(need, W, W.tile, M.ttc_thr, pidx, oidx, kidx, thr);
+            uint32_t pos = 0;
+            const bool got = wq.take(need, W, pos);
             bool ended = false;
             if ((need >> lane) & 1u) {
                 L.active = got;
-                if (got) ended = L.init(M, P, O, pidx, oidx, kidx, thr);
+                if (got) {
+                    const Row rows = row_of(W, pos, M.ttc_thr);
+                    oidx = rows.o;
+                    ended = L.init(M, P, O, rows);
+                }
             }
             need = __ballot_sync(kFull, ended);
         }
@@ -462,9 +466,8 @@ cudaError_t launch_t(const ModelDev &m, const ParamsDev &p, const OutDev &o, con
         if (e != cudaSuccess) return e;
         if (per_sm < 1) per_sm = 1;
     }
-    const uint64_t tiles = tiles_of(w, w.tile);
     uint64_t blocks = (uint64_t)sms * per_sm;
-    uint64_t need_blocks = (tiles + 3) / 4;  // one tile per warp at least
+    const uint64_t need_blocks = (tickets_of(w) + 3) / 4;  // one ticket per warp at least
     if (need_blocks < blocks) blocks = need_blocks;
     if (blocks < 1) blocks = 1;
     kern<<<(unsigned)blocks, 128, 0, s>>>(m, p, o, w);

@@ -132,7 +132,8 @@ struct Wave {
     Clock::time_point t_launch;
     std::vector<ChunkRef> chunks;
     // device and pinned sub-buffers
-    unsigned long long *counter = nullptr;
+    void *scratch = nullptr;  // the rollout's (ticket counter, processing order)
+    size_t scratch_bytes = 0;
     JobDev *djobs = nullptr, *hjobs = nullptr;
     TileDesc *dtiles = nullptr, *htiles = nullptr, *dred = nullptr, *hred = nullptr;
     uint32_t *dfirst = nullptr, *hfirst = nullptr;
@@ -398,7 +399,6 @@ bool aeb_server::launch_wave(Wave &w)
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(w.dfirst, w.hfirst, sizeof(uint32_t) * (nj + 1), cudaMemcpyHostToDevice,
                             w.stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), w.stream);
     if (e == cudaSuccess) {
         ParamsDev pd;
         for (int f = 0; f < AEB_NFIELDS; ++f) pd.col[f] = dcol[f];
@@ -407,9 +407,9 @@ bool aeb_server::launch_wave(Wave &w)
         od.x_ref = dxref;
         od.v_imp = dvimp;
         od.n_steps = dnsteps;
-        WorkDev wd{total, T, w.counter, w.dtiles, nt, w.djobs, 0};
-        e = (cfg.precision == AEB_FP64_PLAIN) ? launch_rollout_fp64(md, pd, od, wd, lcfg, w.stream)
-                                              : launch_rollout_fp32(md, pd, od, wd, lcfg, w.stream);
+        const WorkDev wd{total, T, nullptr, w.dtiles, nt, w.djobs, 0, 0, nullptr};
+        e = launch_rollout(md, pd, cfg.precision, od, wd, w.htiles, lcfg, w.scratch,
+                           w.scratch_bytes, w.stream);
     }
     if (e == cudaSuccess)
         e = launch_reduce_jobs(dstatus, dxref, dvimp, dnsteps, w.dred, nr, w.dfirst, w.djobs, nj,
@@ -616,15 +616,21 @@ extern "C" aeb_status aeb_serve_create(const aeb_serve_cfg *cfg, const aeb_model
     for (auto &w : s->waves) {
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&w.stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming);
-        if (e == cudaSuccess)
-            e = cudaMalloc(&w.dmem, 256 + sz_jobs + sz_tiles + sz_red + sz_first + sz_part + sz_stats);
+        const size_t tables = sz_jobs + sz_tiles + sz_red + sz_first + sz_part + sz_stats;
+        if (e == cudaSuccess) {
+            w.scratch_bytes = rollout_scratch_bytes(max_tiles * T, md, cfg->precision);
+            e = cudaMalloc(&w.dmem, tables + w.scratch_bytes);
+            if (e == cudaErrorMemoryAllocation && w.scratch_bytes > kCounterBytes) {
+                cudaGetLastError();
+                w.scratch_bytes = kCounterBytes;  // no room for a processing order
+                e = cudaMalloc(&w.dmem, tables + w.scratch_bytes);
+            }
+        }
         if (e == cudaSuccess)
             e = cudaHostAlloc(&w.hmem, sz_jobs + sz_tiles + sz_red + sz_first + sz_stats,
                               cudaHostAllocDefault);
         if (e != cudaSuccess) break;
         char *d = static_cast<char *>(w.dmem);
-        w.counter = reinterpret_cast<unsigned long long *>(d);
-        d += 256;
         w.djobs = reinterpret_cast<JobDev *>(d);
         d += sz_jobs;
         w.dtiles = reinterpret_cast<TileDesc *>(d);
@@ -636,6 +642,8 @@ extern "C" aeb_status aeb_serve_create(const aeb_serve_cfg *cfg, const aeb_model
         w.dpart = reinterpret_cast<RedPartial *>(d);
         d += sz_part;
         w.dstats = reinterpret_cast<aeb_job_stats *>(d);
+        d += sz_stats;
+        w.scratch = d;
         char *h = static_cast<char *>(w.hmem);
         w.hjobs = reinterpret_cast<JobDev *>(h);
         h += sz_jobs;

@@ -104,7 +104,7 @@ extern "C" aeb_status aeb_batch_create(const aeb_model *model, const aeb_job *jo
     const size_t o_first = o_red + a256(sizeof(TileDesc) * red.size());
     const size_t o_part = o_first + a256(sizeof(uint32_t) * first.size());
     const size_t o_scratch = o_part + a256(sizeof(RedPartial) * (red.size() + 1));
-    size_t scratch = rollout_scratch_bytes((uint64_t)tiles.size() * T, md, precision);
+    size_t scratch = rollout_scratch_bytes((uint64_t)tiles.size() * T, precision);
 
     aeb_batch *b = new aeb_batch;
     b->device = dev;

@@ -259,17 +259,18 @@ struct Layout {
 // Whether a launch of this many positions is worth ordering.  With at most
 // one warp per sub-partition (152 x 4 x 32 = 19,456 rollouts) a binary32 launch
 // lasts as long as its longest rollout in any order, and the two kernels would
-// add ~10 us to ~200.
-bool wants_order(uint64_t positions)
+// add ~10 us to ~200.  A binary64 warp gains from lanes of one cap class at
+// any size above one warp (its steps take microseconds).
+bool wants_order(uint64_t positions, aeb_precision precision)
 {
-    return positions > 19456;
+    return positions > (precision == AEB_FP64_PLAIN ? 32u : 19456u);
 }
 
 }  // namespace
 
-size_t rollout_scratch_bytes(uint64_t positions, const ModelDev &, aeb_precision)
+size_t rollout_scratch_bytes(uint64_t positions, aeb_precision precision)
 {
-    if (!wants_order(positions)) return kCounterBytes;
+    if (!wants_order(positions, precision)) return kCounterBytes;
     return Layout(std::min(positions, kOrderMax)).bytes;
 }
 
@@ -279,8 +280,8 @@ cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision 
                            cudaStream_t s)
 {
     const uint64_t all = w.tiles ? w.n_tiles * w.tile : w.n;
-    const bool order = m.n_max > 0 && wants_order(all) &&
-                       scratch_bytes >= rollout_scratch_bytes(all, m, precision);
+    const bool order = m.n_max > 0 && wants_order(all, precision) &&
+                       scratch_bytes >= rollout_scratch_bytes(all, precision);
     const uint64_t piece = order ? kOrderMax : kNaturalMax;  // positions per launch
     const uint64_t unit = w.tiles ? piece / w.tile : piece;   // tiles or rows per launch
     const uint64_t total = w.tiles ? w.n_tiles : w.n;

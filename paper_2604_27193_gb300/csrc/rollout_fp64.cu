@@ -32,6 +32,15 @@
 // `tame`); the constants 1, 2, -0, dt and its fractions are kept in registers
 // the compiler cannot take for constants.  51 operations of 64 cycles a step
 // (59 on an axle line) against 57 (65) of 76.
+//
+// A rollout spends most of its steps where r(D) cannot change: before brake
+// onset (a = u = 0), and after it once the demand is on the constant cap, which
+// a growing demand never leaves (icy and wet roads; about half of the
+// single-scenario workload's steps), or with an instantaneous actuator.  A
+// warp whose lanes are all there runs a step without the actuator and with r
+// held: 32 operations (27 and the position) instead of 51.  order.cu hands a
+// warp samples of one cap class and length, so that its lanes are there
+// together.
 #include <climits>
 
 #include "rollout_common.cuh"
@@ -97,6 +106,7 @@ struct Ops {
 
 // Bounds of the states the fused forms are used on: they keep every sum and
 // product of a step below 2^400, so nothing overflows.
+constexpr int kTtcSpan = 256;  // steps one trigger test may cover
 constexpr double kTame = 1e5;
 __device__ __forceinline__ bool tame_speed(double v)  // 0 < v < ~1e5 (false for a NaN)
 {
@@ -131,6 +141,10 @@ struct Lane64 {
     int piece;                    // 0: D, 1, 2: an axle line, 3: the constant cap; -1: none
     bool trig, lagged, ordered;
     bool active;                  // the lane holds a rollout
+    bool damped;                  // dt / tau <= 1: the stage demands approach -a_cmd from below
+    bool held;                    // r is the same at every stage until onset, or for good
+    double nr;                    // -r while held
+    int32_t n_chk;                // TTC: no step before this one can trigger
 
     // Select the line that is the strict minimum at demand D and the demand
     // interval, shrunk by the band, on which it stays so (piece -1 if D is
@@ -196,18 +210,40 @@ struct Lane64 {
     // Realised deceleration r for demand D = -a (Eq. 5 as printed, or the
     // per-axle fixed point min(min(D, mu gc), min(f0 + f1 D, r0 + r1 D))),
     // then dv/dt = -r - k v^2 - g sin(theta) (Eq. 4).
+    __device__ __forceinline__ double realised(double D) const
+    {
+        if (CAP == AEB_CAP_LUMPED) return dmin(D, cap);
+        double lf = f0 + f1 * D;
+        double lr = r0 + r1 * D;
+        return dmin(dmin(D, mg), dmin(lf, lr));
+    }
     __device__ __forceinline__ double accel(double vv, double aa) const
     {
-        double D = -aa;
-        double r;
-        if (CAP == AEB_CAP_LUMPED) {
-            r = dmin(D, cap);
-        } else {
-            double lf = f0 + f1 * D;
-            double lr = r0 + r1 * D;
-            r = dmin(dmin(D, mg), dmin(lf, lr));
-        }
+        const double r = realised(-aa);
         return ((-r) - (k * vv) * vv) - gs;
+    }
+
+    // Hold r at the actuator value aa, at which the lane stays until onset (0)
+    // or for good (an instantaneous actuator's command).
+    __device__ __forceinline__ void hold_at(double aa)
+    {
+        held = ordered;
+        nr = -realised(-aa);
+    }
+
+    // After a step inside a piece, braking: whether the lane is on the constant
+    // cap for good.  The stage demands of a damped lag lie between the present
+    // demand and -a_cmd up to a few ulps (and so do all later ones), and the
+    // constant stays the strict minimum above klo, so it is enough that the
+    // present demand is 2^12 ulps above klo (a positive value) and a >= a_cmd.
+    __device__ __forceinline__ void try_hold(const ModelDev &M)
+    {
+        if (piece == 3 && damped && khi == 0x7ff0000000000000ll &&
+            klo > 0x3f50000000000000ll /* 2^-10 */ && -okey(a) >= klo + 4096 &&
+            okey(a) >= okey(M.a_cmd)) {
+            held = true;
+            nr = (CAP == AEB_CAP_LUMPED) ? -cap : -mg;
+        }
     }
 
     __device__ __forceinline__ int32_t onset() const
@@ -237,6 +273,7 @@ struct Lane64 {
         // (and the sample is inside the range of the fused forms)
         ordered = (!lagged || M.dt * it <= 2.0) && M.dt >= 1e-30 && M.dt <= 1.0 &&
                   fabs(M.a_cmd) <= kTame && k <= 1.0 && fabs(gs) <= kTame;
+        damped = lagged && M.dt * it <= 1.0 && M.a_cmd < 0.0;
         const double mu = f[kMu], gc = f[kGc];
         const double mh = mu * M.hl;
         if (CAP == AEB_CAP_LUMPED) {
@@ -268,11 +305,19 @@ struct Lane64 {
         v = f[kV0];
         a = 0.0;
         n = 0;
+        n_chk = 0;
         select_piece(-a);
+        hold_at(a);
         return false;
     }
 
-    // TTC trigger (while not yet triggered), at the start of step n.
+    // TTC trigger (while not yet triggered), at the start of step n.  A test
+    // that does not fire also bounds the steps that cannot (n_chk): while r is
+    // held the car's acceleration is at most acc = max(0, -r - g sin(theta)),
+    // so over kTtcSpan steps its speed stays below W = v + kTtcSpan dt acc and
+    // the margin (gap + noise) - thr c falls by at most dt (W + |thr| (acc + b_L))
+    // per step (a braking lead's travel only widens the gap; its speed falls by
+    // dt b_L); a reading's noise is at most 3 perc_sigma.
     __device__ __forceinline__ void test_trigger(const ModelDev &M, const Ops &q)
     {
         double gap_meas, closing;
@@ -284,8 +329,10 @@ struct Lane64 {
             gap_meas = q.add(q.sub(d0, x), noise);
             closing = v;
         }
+        const double limit = q.mul(thr, closing);
+        const float margin = (float)(gap_meas - limit) - 3.001f * (float)M.perc_sigma;
         bool reading = true;
-        if (M.perc) {  // the reading of step n + L describes step n
+        if (M.perc && !(margin > 0.0f)) {  // the reading of step n + L describes step n
             uint32_t h[4];
             perc_halves(row, (uint64_t)((long long)n + M.perc_lat), M.perc_seed, h);
             const double s32 = 1.0 / 4294967296.0;  // 2^-32
@@ -294,10 +341,18 @@ struct Lane64 {
             if (u4 < M.perc_drop) reading = false;
             else gap_meas = gap_meas + M.perc_sigma * (2.0 * (((u1 + u2) + u3) - 1.5));
         }
-        if (reading && gap_meas <= thr * closing) {
+        if (reading && gap_meas <= limit) {
             trig = true;
             long long nb = ((long long)n + M.perc_lat) + n_delay;
             n_b = nb > INT_MAX ? INT_MAX : (int32_t)nb;
+        } else if (held && margin > 0.0f && tame_speed(v)) {
+            const float dtf = (float)q.dt, acc = fmaxf(0.0f, (float)(nr - gs));
+            const float W = (float)v + (float)kTtcSpan * dtf * acc;
+            const float fall = dtf * (W + fabsf((float)thr) * (acc + (float)M.lead_decel)) * 1.001f;
+            // margin's own rounding: a few binary32 ulps of what it was formed from
+            const float m = margin * 0.999f - 1e-5f * (fabsf((float)gap_meas) + fabsf((float)limit));
+            const float steps = __fdividef(m, fall);
+            if (steps > 1.0f) n_chk = n + (steps < (float)kTtcSpan ? (int)steps : kTtcSpan);
         }
     }
 
@@ -307,55 +362,73 @@ struct Lane64 {
                                          uint64_t i)
     {
         const double dt = q.dt, h2 = q.h2, h6 = q.h6;
-        if (TTC && active && !trig) test_trigger(M, q);
-        const double u = (trig && n >= n_b) ? M.a_cmd : 0.0;
-
-        double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
-        if (lagged) {
-            a1 = a;
-            ka1 = q.mul(q.sub(u, a1), it);
-            a2 = q.add(a, q.mul(h2, ka1));
-            ka2 = q.mul(q.sub(u, a2), it);
-            a3 = q.add(a, q.mul(h2, ka2));
-            ka3 = q.mul(q.sub(u, a3), it);
-            a4 = q.add(a, q.mul(dt, ka3));
-            ka4 = q.mul(q.sub(u, a4), it);
-        } else {
-            a1 = a2 = a3 = a4 = u;
+        if (TTC && active && !trig && n >= n_chk) test_trigger(M, q);
+        if (trig && n == n_b) {  // the command switches on: a moves from here, or has moved
+            held = false;
+            if (!lagged) hold_at(M.a_cmd);
         }
-        // With dt / tau <= 2 the stage demands lie between the first and the
-        // fourth (-a1 smallest when the command is a deceleration, so that
-        // a - u >= 0 from the start, -a4 smallest otherwise): two tests for
-        // the step.
-        // (A piece exists only when dt / tau <= 2, where the lag is stable and
-        // the stage actuator values are finite, so order keys compare them.)
-        const bool dec = M.a_cmd <= 0.0;
-        const long long kfirst = -okey(dec ? a1 : a4), klast = -okey(dec ? a4 : a1);
-        const bool pw = piece >= 0 && kfirst >= klo && klast <= khi && tame_speed(v);
-        const bool lines = __any_sync(kFull, active && pw && (piece == 1 || piece == 2));
+        const bool braking = trig && n >= n_b;
+        const double u = braking ? M.a_cmd : 0.0;
         double v2, v3, v4, xn, vn, an;
-        if (pw) {
-            const double kv1 = accel_piece(q, v, a1, lines);
+        bool pw = true;
+        if (__all_sync(kFull, !active || (held && tame_speed(v)))) {
+            const double kv1 = q.sub(q.sub(nr, q.mul(q.mul(k, v), v)), gs);
             v2 = q.add(v, q.mul(h2, kv1));
-            const double kv2 = accel_piece(q, v2, a2, lines);
+            const double kv2 = q.sub(q.sub(nr, q.mul(q.mul(k, v2), v2)), gs);
             v3 = q.add(v, q.mul(h2, kv2));
-            const double kv3 = accel_piece(q, v3, a3, lines);
+            const double kv3 = q.sub(q.sub(nr, q.mul(q.mul(k, v3), v3)), gs);
             v4 = q.add(v, q.mul(dt, kv3));
-            const double kv4 = accel_piece(q, v4, a4, lines);
+            const double kv4 = q.sub(q.sub(nr, q.mul(q.mul(k, v4), v4)), gs);
             xn = q.combine(x, v, v2, v3, v4);
             vn = q.combine(v, kv1, kv2, kv3, kv4);
-            an = lagged ? q.combine(a, ka1, ka2, ka3, ka4) : u;
-        } else if (active) {
-            const double kv1 = accel(v, a1);
-            v2 = v + h2 * kv1;
-            const double kv2 = accel(v2, a2);
-            v3 = v + h2 * kv2;
-            const double kv3 = accel(v3, a3);
-            v4 = v + dt * kv3;
-            const double kv4 = accel(v4, a4);
-            xn = x + h6 * (((v + 2.0 * v2) + 2.0 * v3) + v4);
-            vn = v + h6 * (((kv1 + 2.0 * kv2) + 2.0 * kv3) + kv4);
-            an = lagged ? a + h6 * (((ka1 + 2.0 * ka2) + 2.0 * ka3) + ka4) : u;
+            an = lagged ? a : u;  // not read while r is held
+        } else {
+            double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
+            if (lagged) {
+                a1 = a;
+                ka1 = q.mul(q.sub(u, a1), it);
+                a2 = q.add(a, q.mul(h2, ka1));
+                ka2 = q.mul(q.sub(u, a2), it);
+                a3 = q.add(a, q.mul(h2, ka2));
+                ka3 = q.mul(q.sub(u, a3), it);
+                a4 = q.add(a, q.mul(dt, ka3));
+                ka4 = q.mul(q.sub(u, a4), it);
+            } else {
+                a1 = a2 = a3 = a4 = u;
+            }
+            // With dt / tau <= 2 the stage demands lie between the first and the
+            // fourth (-a1 smallest when the command is a deceleration, so that
+            // a - u >= 0 from the start, -a4 smallest otherwise): two tests for
+            // the step.
+            // (A piece exists only when dt / tau <= 2, where the lag is stable and
+            // the stage actuator values are finite, so order keys compare them.)
+            const bool dec = M.a_cmd <= 0.0;
+            const long long kfirst = -okey(dec ? a1 : a4), klast = -okey(dec ? a4 : a1);
+            pw = piece >= 0 && kfirst >= klo && klast <= khi && tame_speed(v);
+            const bool lines = __any_sync(kFull, active && pw && (piece == 1 || piece == 2));
+            if (pw) {
+                const double kv1 = accel_piece(q, v, a1, lines);
+                v2 = q.add(v, q.mul(h2, kv1));
+                const double kv2 = accel_piece(q, v2, a2, lines);
+                v3 = q.add(v, q.mul(h2, kv2));
+                const double kv3 = accel_piece(q, v3, a3, lines);
+                v4 = q.add(v, q.mul(dt, kv3));
+                const double kv4 = accel_piece(q, v4, a4, lines);
+                xn = q.combine(x, v, v2, v3, v4);
+                vn = q.combine(v, kv1, kv2, kv3, kv4);
+                an = lagged ? q.combine(a, ka1, ka2, ka3, ka4) : u;
+            } else if (active) {
+                const double kv1 = accel(v, a1);
+                v2 = v + h2 * kv1;
+                const double kv2 = accel(v2, a2);
+                v3 = v + h2 * kv2;
+                const double kv3 = accel(v3, a3);
+                v4 = v + dt * kv3;
+                const double kv4 = accel(v4, a4);
+                xn = x + h6 * (((v + 2.0 * v2) + 2.0 * v3) + v4);
+                vn = v + h6 * (((kv1 + 2.0 * kv2) + 2.0 * kv3) + kv4);
+                an = lagged ? a + h6 * (((ka1 + 2.0 * ka2) + 2.0 * ka3) + ka4) : u;
+            }
         }
         if (!active) return false;
 
@@ -391,6 +464,7 @@ struct Lane64 {
         a = an;
         n = n + 1;
         if (!pw) select_piece(-a);
+        else if (braking && !held) try_hold(M);
         return false;
     }
 };
@@ -428,7 +502,9 @@ k_rollout_fp64(ModelDev M, ParamsDev P, OutDev O, WorkDev W)
     L.row = 0;
     L.n = L.n_b = L.n_delay = 0;
     L.piece = -1;
-    L.trig = L.lagged = L.ordered = false;
+    L.trig = L.lagged = L.ordered = L.damped = L.held = false;
+    L.nr = 0.0;
+    L.n_chk = 0;
     uint64_t oidx = 0;
     unsigned need = kFull;
     for (;;) {

@@ -101,6 +101,18 @@ enum { K_RUN = 0, K_INVALID, K_CONTACT0, K_STOP0, K_HORIZON0 };
 // lead pays nothing for the moving one).
 enum { kNoLead = 0, kLeadStationary = 1, kLeadMoving = 2 };
 
+// What a step takes r + g sin(theta) from: the current piece of r(D), the full
+// minimum, or the constant C (every a_j zero).
+enum { kStepPiece, kStepFullMin, kStepFlat };
+// Steps per trip of a full window.  The kernels' code competes for the
+// instruction caches: both bodies unrolled over the whole window (32) are 1-5 %
+// slower than 16 steps of the piece body and 8 of the flat one (single
+// scenario 1e6 2.44 against 2.40 ms, 2e5 at 0.1 ms 5.3 against 5.0, grid of 216
+// jobs 6.61 against 6.40); 8 or 4 of either are within 1 % of those.
+constexpr int kPieceUnroll = 16, kFlatUnroll = 8;
+static_assert(AEB_FP32_WINDOW % kPieceUnroll == 0 && AEB_FP32_WINDOW % kFlatUnroll == 0,
+              "whole trips per window");
+
 struct ModelF32 {
     float acmd;
     // binary32 copies of the constants the tile preparation forms binary32
@@ -387,7 +399,7 @@ struct Lane32 {
     // formed as 6 v1 + s dt (q1 + q2 + q3) (the same sum in exact arithmetic,
     // one instruction fewer).  Returns the end-of-step low words and actuator
     // deviation.
-    template <bool FULL_MIN>
+    template <int KIND>
     __device__ __forceinline__ void rk4_step(float &vl1, float &gl1, float &en) const
     {
         const float v1 = vh + vl;
@@ -395,7 +407,9 @@ struct Lane32 {
         // of the stage chain: two paired binary32 FMAs (per component the same
         // rounding as fmaf) cost two issue slots instead of four
         float2 X12, X34;
-        if (FULL_MIN) {
+        if (KIND == kStepFlat) {
+            X12 = X34 = make_float2(C, C);
+        } else if (KIND == kStepFullMin) {
             X12 = make_float2(rg_full(np1()), rg_full(cf(L_NP2)));
             X34 = make_float2(rg_full(cf(L_NP3)), rg_full(cf(L_NP4)));
         } else {
@@ -469,6 +483,13 @@ struct Lane32 {
         n = n + 1;
     }
 
+    // Whether r + g sin(theta) is C at every stage whatever e: before onset, on
+    // the constant cap, or with an instantaneous actuator (a_j = +-0).
+    __device__ __forceinline__ bool flat() const
+    {
+        return a1 == 0.0f && a2 == 0.0f && a3 == 0.0f && a4 == 0.0f;
+    }
+
     // A checked step inside the current piece; true if the rollout ended
     // (contact or stop) in this step, which is then not committed (its
     // end-of-step low words are returned).
@@ -476,17 +497,18 @@ struct Lane32 {
                                               float sig)
     {
         float en;
-        rk4_step<false>(vl1, gl1, en);
+        rk4_step<kStepPiece>(vl1, gl1, en);
         const bool ended = terminal(F, vl1, gl1, sig);
         if (!ended) commit(vl1, gl1, en);
         return ended;
     }
 
     // An unchecked step inside the current piece (step counter not advanced).
+    template <int KIND>
     __device__ __forceinline__ void step_unchecked()
     {
         float vl1, gl1, en;
-        rk4_step<false>(vl1, gl1, en);
+        rk4_step<KIND>(vl1, gl1, en);
         vl = vl1;
         gl = gl1;
         e = en;
@@ -546,23 +568,29 @@ struct Lane32 {
     // different lengths run the same window code, each masked off after its
     // own length (the short-window version is a rolled loop, to keep the
     // kernel's code small).
-    template <bool FULL>
+    // FLAT: every lane of the warp is flat(); the actuator terms are C.
+    template <bool FULL, bool FLAT>
     __device__ __forceinline__ bool step_window(const ModelF32 &F, int len)
     {
+        constexpr int KIND = FLAT ? kStepFlat : kStepPiece;
         const float vh0 = vh, vl0 = vl, gh0 = gh, gl0 = gl, e0 = e;
         if (FULL) {
             len = AEB_FP32_WINDOW;
+            constexpr int kTrip = FLAT ? kFlatUnroll : kPieceUnroll;
+#pragma unroll 1
+            for (int t = 0; t < AEB_FP32_WINDOW; t += kTrip) {
 #pragma unroll
-            for (int j = 0; j < AEB_FP32_WINDOW; ++j) step_unchecked();
+                for (int j = 0; j < kTrip; ++j) step_unchecked<KIND>();
+            }
         } else {
             // rolled (code size), two steps per trip, then the odd step
             int j = 0;
 #pragma unroll 1
             for (; j + 2 <= len; j += 2) {
-                step_unchecked();
-                step_unchecked();
+                step_unchecked<KIND>();
+                step_unchecked<KIND>();
             }
-            if (j < len) step_unchecked();
+            if (j < len) step_unchecked<KIND>();
         }
         normalize();
         bool hit = vh <= 0.0f;
@@ -602,7 +630,7 @@ struct Lane32 {
             e = e - F.acmd;
         }
         float en;
-        rk4_step<true>(vl1, gl1, en);
+        rk4_step<kStepFullMin>(vl1, gl1, en);
         const bool ended = terminal(F, vl1, gl1, cf(L_SIGMA)) || n >= n_last;
         if (!ended) {
             commit(vl1, gl1, en);
@@ -764,19 +792,19 @@ struct Lane32 {
                 st[j] = gl;
                 st[AEB_FP32_WINDOW + j] = vl;
             }
-            step_unchecked();
+            step_unchecked<kStepPiece>();
             if (st) {
                 st[j + 1] = gl;
                 st[AEB_FP32_WINDOW + j + 1] = vl;
             }
-            step_unchecked();
+            step_unchecked<kStepPiece>();
         }
         if (j < len) {
             if (st) {
                 st[j] = gl;
                 st[AEB_FP32_WINDOW + j] = vl;
             }
-            step_unchecked();
+            step_unchecked<kStepPiece>();
         }
         normalize();
         bool hit = vh <= 0.0f;
@@ -1224,7 +1252,16 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
             // (the perception kernels, whose readings and band code already
             // fill the instruction cache, run it through the rolled loop: the
             // unrolled copy costs them more in cache misses than it saves)
-            if (active) replay = L.template step_window<!PERC>(F, len);
+            // A warp whose lanes are all flat (order.cu hands a warp samples of
+            // one cap class) drops the actuator terms: 16 instructions a step
+            // on 16 FMA-pipe slots instead of 18 on 20 (icy roads 2.31 -> 2.03
+            // ms per 1e6).  Short windows keep the one body (a second costs
+            // what it gains).
+            if (__all_sync(kFull, !active || L.flat())) {
+                if (active) replay = L.template step_window<!PERC, true>(F, len);
+            } else {
+                if (active) replay = L.template step_window<!PERC, false>(F, len);
+            }
         } else if (PERC && __any_sync(kFull, slot >= 0)) {
             // Band lanes keep their window's states; then the warp tests each
             // band lane's trigger at all the window's steps at once (lane j:
@@ -1275,7 +1312,7 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
                 }
             }
         } else {
-            if (active && len > 0) replay = L.template step_window<false>(F, len);
+            if (active && len > 0) replay = L.template step_window<false, false>(F, len);
         }
         // Slow steps (breakpoint crossings, the horizon's last step) after the
         // windows: a window that stopped right before one takes it in the same

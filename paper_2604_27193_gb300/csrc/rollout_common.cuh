@@ -79,44 +79,6 @@ __host__ __forceinline__ uint64_t tickets_of(const WorkDev &w)
     return (w.tiles && !w.perm) ? w.n_tiles : (w.n + w.tile - 1) / w.tile;
 }
 
-// A warp's cursor into its ticket.  All 32 lanes call take() together with the
-// same `need` mask (the lanes whose rollout just ended).  Each lane in `need`
-// receives the position of the next unclaimed sample of the warp's ticket;
-// when it is used up the warp claims the next.  Lanes get false once every
-// ticket has been claimed.  Per-sample results never depend on which warp runs
-// a sample.
-struct WarpQueue {
-    Ticket cur{0, 0, false};
-    int used = 0;
-    bool dry = false;
-
-    __device__ __forceinline__ bool take(unsigned need, const WorkDev &w, uint32_t &pos)
-    {
-        const unsigned lane = threadIdx.x & 31u;
-        bool mine = false;
-        while (need && !dry) {
-            if (used >= cur.count) {
-                cur = claim_ticket(w);
-                used = 0;
-                if (!cur.ok) {
-                    dry = true;
-                    break;
-                }
-            }
-            const unsigned rank = __popc(need & lanemask_lt());
-            const bool got = ((need >> lane) & 1u) && (int)rank < cur.count - used;
-            if (got) {
-                mine = true;
-                pos = position(w, cur.start + used + rank);
-            }
-            const unsigned taken = __ballot_sync(kFull, got);
-            used += __popc(taken);
-            need &= ~taken;
-        }
-        return mine;
-    }
-};
-
 // Philox-4x64-10 (Salmon, Moraes, Dror, Shaw, SC 2011): the block of counter
 // c under key (k0, k1), in place.  Used for the per-step perception readings
 // of the TTC trigger, two readings per block: counter (parameter row,

@@ -129,15 +129,167 @@ __device__ __forceinline__ double lead_speed(const ModelDev &M, double t)
     return M.lead_v0 - M.lead_decel * t;
 }
 
+// Realised deceleration r for demand D = -a (Eq. 5 as printed, or the per-axle
+// fixed point min(min(D, mu gc), min(f0 + f1 D, r0 + r1 D)); c: the constant cap).
+template <int CAP>
+__device__ __forceinline__ double realised(double f0, double f1, double r0, double r1, double c,
+                                           double D)
+{
+    if (CAP == AEB_CAP_LUMPED) return dmin(D, c);
+    double lf = f0 + f1 * D;
+    double lr = r0 + r1 * D;
+    return dmin(dmin(D, c), dmin(lf, lr));
+}
+
+// A warp's shared memory: the prepared samples of (up to 32 of) its ticket, and
+// each lane's rarely read values in a column of its own.
+enum { S_V0, S_D0, S_GS, S_K, S_IT, S_KEY, S_NCOPY,  // KEY: perception-key row, as bits
+       S_F0 = S_NCOPY, S_F1, S_R0, S_R1, S_MG, S_NOISE, S_THR, S_N };
+enum { K_F0, K_F1, K_R0, K_R1, K_MG, K_NOISE, K_THR, K_N };  // S_F0 + K_*
+enum { B_RUN = 1, B_LAGGED = 2, B_ORDERED = 4, B_DAMPED = 8 };
+struct WarpMem {
+    double rec[S_N][32];
+    double cold[K_N][32];
+    float line[5][32], cline[5][32];  // f0, f1, r0, r1, mg (or cap) in binary32
+    uint32_t pos[32];
+    int32_t delay[32], bits[32];
+};
+
+// The line of r(D) that is the strict minimum at D and the demand interval, as
+// order keys, on which it stays so (piece -1: none can be named).
+struct Piece {
+    int piece;
+    long long klo, khi;
+};
+
+// In binary64: the interval shrunk by a band of 1e-12 relative.
+__device__ __noinline__ Piece select_exact(bool lumped, double f0, double f1, double r0,
+                                           double r1, double c, double D)
+{
+    Piece p{-1, 0, 0};
+    const double A[4] = {0.0, lumped ? c : f0, r0, c};
+    const double S[4] = {1.0, lumped ? 0.0 : f1, r1, 0.0};
+    const int nl = lumped ? 2 : 4;
+    double val[4];
+    int cur = 0;
+    for (int j = 0; j < nl; ++j) {
+        val[j] = (j == 0) ? D : A[j] + S[j] * D;
+        if (val[j] < val[cur]) cur = j;
+    }
+    double lo = -dinf(), hi = dinf();
+    for (int j = 0; j < nl; ++j) {
+        if (j == cur) continue;
+        const double ds = S[cur] - S[j];
+        if (!(fabs(ds) >= 1e-6) || !(val[j] > val[cur])) return p;
+        const double B = (A[j] - A[cur]) / ds;  // line j meets the current line
+        const double band = 1e-12 * (1.0 + fabs(A[j]) + fabs(A[cur]) + fabs(B)) / fabs(ds);
+        if (ds > 0.0) hi = fmin(hi, B - band);  // line j is below beyond B
+        else lo = fmax(lo, B + band);
+    }
+    if (!(lo <= D && D <= hi)) return p;
+    p.klo = okey(lo);
+    p.khi = okey(hi);
+    p.piece = (lumped && cur == 1) ? 3 : cur;
+    return p;
+}
+
+// In binary32, for demands that are not close to a breakpoint (binary64
+// divisions cost ~1000 cycles each): the same with a band of 1e-5 relative
+// (all slopes at most 8, at least 1e-3 apart), far above the rounding of the
+// lines and of their crossings, so the line is the strict minimum on the
+// interval in binary64 too.
+__device__ __forceinline__ Piece select_fast(bool lumped, const float (*ln)[32], int lane, float D)
+{
+    Piece p{-1, 0, 0};
+    const float c = ln[4][lane];
+    const float A[4] = {0.0f, lumped ? c : ln[0][lane], ln[2][lane], c};
+    const float S[4] = {1.0f, lumped ? 0.0f : ln[1][lane], ln[3][lane], 0.0f};
+    const int nl = lumped ? 2 : 4;
+    float cv = D, cA = 0.0f, cS = 1.0f;
+    int cur = 0;
+#pragma unroll
+    for (int j = 1; j < 4; ++j) {
+        if (j >= nl) continue;
+        const float vj = fmaf(S[j], D, A[j]);
+        if (vj < cv) {
+            cv = vj;
+            cA = A[j];
+            cS = S[j];
+            cur = j;
+        }
+    }
+    const float inf = __int_as_float(0x7f800000);
+    float lo = -inf, hi = inf;
+    bool ok = fabsf(cS) <= 8.0f && fabsf(cA) < 1e6f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (j >= nl || j == cur) continue;
+        const float ds = cS - S[j];
+        ok = ok && fabsf(ds) >= 1e-3f && fabsf(S[j]) <= 8.0f && fabsf(A[j]) < 1e6f;
+        const float B = __fdividef(A[j] - cA, ds);
+        const float band = __fdividef(1e-5f * (1.0f + fabsf(A[j]) + fabsf(cA) + fabsf(B)), fabsf(ds));
+        if (ds > 0.0f) hi = fminf(hi, B - band);
+        else lo = fmaxf(lo, B + band);
+    }
+    const float slack = 1e-6f * (1.0f + fabsf(D));  // D's own rounding
+    if (!ok || !(lo + slack <= D && D + slack <= hi)) return p;
+    p.klo = okey((double)lo);
+    p.khi = okey((double)hi);
+    p.piece = (lumped && cur == 1) ? 3 : cur;
+    return p;
+}
+
+// A step by the plain expressions of the definition, for states outside the
+// range of the fused forms or without ordered stage demands.
+struct Plain {
+    double x, v, a;
+};
+template <int CAP>
+__device__ __noinline__ Plain plain_step(double x, double v, double a, double u, double it,
+                                         bool lagged, double k, double gs, double f0, double f1,
+                                         double r0, double r1, double c, double dt, double h2,
+                                         double h6)
+{
+    double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
+    if (lagged) {
+        a1 = a;
+        ka1 = (u - a1) * it;
+        a2 = a + h2 * ka1;
+        ka2 = (u - a2) * it;
+        a3 = a + h2 * ka2;
+        ka3 = (u - a3) * it;
+        a4 = a + dt * ka3;
+        ka4 = (u - a4) * it;
+    } else {
+        a1 = a2 = a3 = a4 = u;
+    }
+    auto accel = [&](double vv, double aa) {
+        const double r = realised<CAP>(f0, f1, r0, r1, c, -aa);
+        return ((-r) - (k * vv) * vv) - gs;
+    };
+    const double kv1 = accel(v, a1);
+    const double v2 = v + h2 * kv1;
+    const double kv2 = accel(v2, a2);
+    const double v3 = v + h2 * kv2;
+    const double kv3 = accel(v3, a3);
+    const double v4 = v + dt * kv3;
+    const double kv4 = accel(v4, a4);
+    Plain p;
+    p.x = x + h6 * (((v + 2.0 * v2) + 2.0 * v3) + v4);
+    p.v = v + h6 * (((kv1 + 2.0 * kv2) + 2.0 * kv3) + kv4);
+    p.a = lagged ? a + h6 * (((ka1 + 2.0 * ka2) + 2.0 * ka3) + ka4) : u;
+    return p;
+}
+
 template <int CAP, bool LEAD, bool TTC>
 struct Lane64 {
     double x, v, a;
-    double d0, gs, noise, k, it, thr;
-    double mg, f0, f1, r0, r1, cap;
+    double d0, gs, k, it;
+    double c;                     // the constant cap: mu g cos(theta), or the Eq. 5 cap
     double pa, pb;                // current line pa + pb D (piece 1, 2)
     long long klo, khi;           // its demand interval [dlo, dhi] as order keys
-    uint64_t row;                 // perception key row (counter of the readings)
     int32_t n, n_b, n_delay;
+    uint32_t pos;
     int piece;                    // 0: D, 1, 2: an axle line, 3: the constant cap; -1: none
     bool trig, lagged, ordered;
     bool active;                  // the lane holds a rollout
@@ -145,90 +297,63 @@ struct Lane64 {
     bool held;                    // r is the same at every stage until onset, or for good
     double nr;                    // -r while held
     int32_t n_chk;                // TTC: no step before this one can trigger
+    WarpMem *mem;
+    int lane;
 
-    // Select the line that is the strict minimum at demand D and the demand
-    // interval, shrunk by the band, on which it stays so (piece -1 if D is
-    // inside a band, lines are nearly parallel, or the stage demands are not
-    // ordered).
-    __device__ void select_piece(double D)
+    __device__ __forceinline__ double cold(int f) const { return mem->cold[f][lane]; }
+
+    __device__ __forceinline__ void select_piece(double D)
     {
         piece = -1;
         if (!ordered) return;
-        double A[4], S[4];
-        int nl;
-        if (CAP == AEB_CAP_LUMPED) {
-            A[0] = 0.0; S[0] = 1.0; A[1] = cap; S[1] = 0.0;
-            nl = 2;
-        } else {
-            A[0] = 0.0; S[0] = 1.0; A[1] = f0; S[1] = f1; A[2] = r0; S[2] = r1; A[3] = mg; S[3] = 0.0;
-            nl = 4;
-        }
-        double val[4];
-        int cur = 0;
-        for (int j = 0; j < nl; ++j) {
-            val[j] = (j == 0) ? D : A[j] + S[j] * D;
-            if (val[j] < val[cur]) cur = j;
-        }
-        double lo = -dinf(), hi = dinf();
-        for (int j = 0; j < nl; ++j) {
-            if (j == cur) continue;
-            const double ds = S[cur] - S[j];
-            if (!(fabs(ds) >= 1e-6) || !(val[j] > val[cur])) return;
-            const double B = (A[j] - A[cur]) / ds;  // line j meets the current line
-            const double band = 1e-12 * (1.0 + fabs(A[j]) + fabs(A[cur]) + fabs(B)) / fabs(ds);
-            if (ds > 0.0) hi = fmin(hi, B - band);  // line j is below beyond B
-            else lo = fmax(lo, B + band);
-        }
-        if (!(lo <= D && D <= hi)) return;
-        if (!(fabs(A[cur]) < 1e50 && fabs(S[cur]) < 1e50)) return;  // see Ops
-        klo = okey(lo);
-        khi = okey(hi);
-        if (CAP == AEB_CAP_LUMPED) {
-            piece = (cur == 0) ? 0 : 3;
-        } else {
-            piece = cur;
-            pa = A[cur];
-            pb = S[cur];
+        Piece p = select_fast(CAP == AEB_CAP_LUMPED, mem->cline, lane, (float)D);
+        if (p.piece < 0)
+            p = select_exact(CAP == AEB_CAP_LUMPED, cold(K_F0), cold(K_F1), cold(K_R0),
+                             cold(K_R1), c, D);
+        piece = p.piece;
+        klo = p.klo;
+        khi = p.khi;
+        if (CAP != AEB_CAP_LUMPED && piece >= 0) {
+            pa = cold(piece == 2 ? K_R0 : K_F0);
+            pb = cold(piece == 2 ? K_R1 : K_F1);
         }
     }
 
-    // dv/dt on the current piece: the same value as `accel` for D in the
-    // piece's interval.  `lines`: some lane of the warp is on an axle line.
-    __device__ __forceinline__ double accel_piece(const Ops &q, double vv, double aa,
-                                                  bool lines) const
+    // dv/dt from -r: (-r - (k v) v) - g sin(theta).
+    __device__ __forceinline__ double accel(const Ops &q, double vv, double mr) const
     {
-        const double D = -aa;
-        const double c = (CAP == AEB_CAP_LUMPED) ? cap : mg;
-        double r = (piece == 0) ? D : c;
+        return q.sub(q.sub(mr, q.mul(q.mul(k, vv), vv)), gs);
+    }
+    // -r on the current piece (or held): the same value as the full minimum's
+    // for a demand -aa in the piece's interval.  `lines`: some lane of the warp
+    // is on an axle line.
+    __device__ __forceinline__ double r_piece(const Ops &q, double aa, bool lines) const
+    {
+        double mr = (piece == 0) ? aa : -c;
         if (CAP != AEB_CAP_LUMPED && lines) {
-            const double rl = q.add(pa, q.mul(pb, D));
-            if (piece == 1 || piece == 2) r = rl;
+            const double rl = q.add(pa, q.mul(pb, -aa));
+            if (piece == 1 || piece == 2) mr = -rl;
         }
-        return q.sub(q.sub(-r, q.mul(q.mul(k, vv), vv)), gs);
+        return held ? nr : mr;
     }
-
-    // Realised deceleration r for demand D = -a (Eq. 5 as printed, or the
-    // per-axle fixed point min(min(D, mu gc), min(f0 + f1 D, r0 + r1 D))),
-    // then dv/dt = -r - k v^2 - g sin(theta) (Eq. 4).
-    __device__ __forceinline__ double realised(double D) const
+    // -r by the full minimum in fused forms (finite lines; order keys compare
+    // as the values).
+    __device__ __forceinline__ double r_full(const Ops &q, double aa) const
     {
-        if (CAP == AEB_CAP_LUMPED) return dmin(D, cap);
-        double lf = f0 + f1 * D;
-        double lr = r0 + r1 * D;
-        return dmin(dmin(D, mg), dmin(lf, lr));
-    }
-    __device__ __forceinline__ double accel(double vv, double aa) const
-    {
-        const double r = realised(-aa);
-        return ((-r) - (k * vv) * vv) - gs;
+        auto kmin = [](double a, double b) { return okey(b) < okey(a) ? b : a; };
+        const double D = -aa;
+        if (CAP == AEB_CAP_LUMPED) return held ? nr : -kmin(D, c);
+        const double lf = q.add(cold(K_F0), q.mul(cold(K_F1), D));
+        const double lr = q.add(cold(K_R0), q.mul(cold(K_R1), D));
+        return held ? nr : -kmin(kmin(D, c), kmin(lf, lr));
     }
 
     // Hold r at the actuator value aa, at which the lane stays until onset (0)
-    // or for good (an instantaneous actuator's command).
+    // or for good (an instantaneous or settled actuator's command).
     __device__ __forceinline__ void hold_at(double aa)
     {
         held = ordered;
-        nr = -realised(-aa);
+        nr = -realised<CAP>(cold(K_F0), cold(K_F1), cold(K_R0), cold(K_R1), c, -aa);
     }
 
     // After a step inside a piece, braking: whether the lane is on the constant
@@ -242,7 +367,9 @@ struct Lane64 {
             klo > 0x3f50000000000000ll /* 2^-10 */ && -okey(a) >= klo + 4096 &&
             okey(a) >= okey(M.a_cmd)) {
             held = true;
-            nr = (CAP == AEB_CAP_LUMPED) ? -cap : -mg;
+            nr = -c;
+        } else if (__double_as_longlong(a) == __double_as_longlong(M.a_cmd)) {
+            hold_at(a);  // settled: a does not move any more
         }
     }
 
@@ -251,64 +378,35 @@ struct Lane64 {
         return TTC ? (trig ? n_b : -1) : n_delay;
     }
 
-    __device__ __forceinline__ bool init(const ModelDev &M, const ParamsDev &P,
-                                         const OutDev &O, const Row &rows)
+    // Take the prepared sample `slot`.
+    __device__ __forceinline__ void take(int slot)
     {
-        double f[AEB_NFIELDS];
-        const uint64_t i = rows.o;
-        load_fields(P, rows.p, f);
-        thr = rows.thr;
-        if (!sample_valid(f)) {
-            const double nan = __longlong_as_double(0x7ff8000000000000ll);
-            store_out(O, i, AEB_INVALID, nan, nan, nan, nan, 0, -1);
-            return true;
-        }
-        row = rows.k;
-        d0 = f[kD0];
-        gs = f[kGs];
-        noise = f[kNoise];
-        k = ((M.rho * f[kCd]) * M.area) / (2.0 * f[kMass]);
-        lagged = f[kTau] > 0.0;
-        it = lagged ? 1.0 / f[kTau] : 0.0;
-        // (and the sample is inside the range of the fused forms)
-        ordered = (!lagged || M.dt * it <= 2.0) && M.dt >= 1e-30 && M.dt <= 1.0 &&
-                  fabs(M.a_cmd) <= kTame && k <= 1.0 && fabs(gs) <= kTame;
-        damped = lagged && M.dt * it <= 1.0 && M.a_cmd < 0.0;
-        const double mu = f[kMu], gc = f[kGc];
-        const double mh = mu * M.hl;
-        if (CAP == AEB_CAP_LUMPED) {
-            cap = (mu * M.g) / (1.0 + mh);
-        } else {
-            mg = mu * gc;
-            f0 = (mg * M.phi_f) / (1.0 - mh);
-            f1 = (1.0 - M.beta) / (1.0 - mh);
-            r0 = (mg * (1.0 - M.phi_f)) / (1.0 + mh);
-            r1 = M.beta / (1.0 + mh);
-        }
-        n_delay = steps_to_reach_dev(f[kTdelay], M.dt);
+        const WarpMem &w = *mem;
+        v = w.rec[S_V0][slot];
+        d0 = w.rec[S_D0][slot];
+        gs = w.rec[S_GS][slot];
+        k = w.rec[S_K][slot];
+        it = w.rec[S_IT][slot];
+        c = w.rec[S_MG][slot];
+#pragma unroll
+        for (int f = 0; f < K_N; ++f) mem->cold[f][lane] = w.rec[S_F0 + f][slot];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) mem->cline[f][lane] = w.line[f][slot];
+        if (TTC) mem->cold[K_MG][lane] = w.rec[S_KEY][slot];  // (c is in a register)
+        pos = w.pos[slot];
+        n_delay = w.delay[slot];
+        const int b = w.bits[slot];
+        lagged = b & B_LAGGED;
+        ordered = b & B_ORDERED;
+        damped = b & B_DAMPED;
         trig = !TTC;
         n_b = n_delay;
-        const int32_t on = TTC ? -1 : n_delay;
-        if (LEAD && d0 <= 0.0) {
-            store_out(O, i, AEB_CONTACT, 0.0, 0.0, f[kV0], 0.0, 0, on);
-            return true;
-        }
-        if (f[kV0] <= 0.0) {
-            store_out(O, i, AEB_STOP, 0.0, 0.0, 0.0, 0.0, 0, on);
-            return true;
-        }
-        if (M.n_max == 0) {
-            store_out(O, i, AEB_HORIZON, 0.0, 0.0, 0.0, 0.0, 0, on);
-            return true;
-        }
         x = 0.0;
-        v = f[kV0];
         a = 0.0;
         n = 0;
         n_chk = 0;
         select_piece(-a);
         hold_at(a);
-        return false;
     }
 
     // TTC trigger (while not yet triggered), at the start of step n.  A test
@@ -323,18 +421,19 @@ struct Lane64 {
         double gap_meas, closing;
         if (M.lead_moving) {  // gap and closing speed to the moving lead
             const double t = from_int(n) * q.dt;
-            gap_meas = ((d0 + lead_pos(M, t)) - x) + noise;
+            gap_meas = ((d0 + lead_pos(M, t)) - x) + cold(K_NOISE);
             closing = v - lead_speed(M, t);
         } else {
-            gap_meas = q.add(q.sub(d0, x), noise);
+            gap_meas = q.add(q.sub(d0, x), cold(K_NOISE));
             closing = v;
         }
+        const double thr = cold(K_THR);
         const double limit = q.mul(thr, closing);
         const float margin = (float)(gap_meas - limit) - 3.001f * (float)M.perc_sigma;
         bool reading = true;
         if (M.perc && !(margin > 0.0f)) {  // the reading of step n + L describes step n
             uint32_t h[4];
-            perc_halves(row, (uint64_t)((long long)n + M.perc_lat), M.perc_seed, h);
+            perc_halves((uint64_t)__double_as_longlong(cold(K_MG)), (uint64_t)((long long)n + M.perc_lat), M.perc_seed, h);
             const double s32 = 1.0 / 4294967296.0;  // 2^-32
             const double u1 = (double)h[0] * s32, u2 = (double)h[1] * s32;
             const double u3 = (double)h[2] * s32, u4 = (double)h[3] * s32;
@@ -359,7 +458,7 @@ struct Lane64 {
     // One RK4 step (all lanes of the warp together); true if the lane's rollout
     // ended (stored).
     __device__ __forceinline__ bool step(const ModelDev &M, const Ops &q, const OutDev &O,
-                                         uint64_t i)
+                                         const WorkDev &W)
     {
         const double dt = q.dt, h2 = q.h2, h6 = q.h6;
         if (TTC && active && !trig && n >= n_chk) test_trigger(M, q);
@@ -369,69 +468,83 @@ struct Lane64 {
         }
         const bool braking = trig && n >= n_b;
         const double u = braking ? M.a_cmd : 0.0;
+        const bool fused = ordered && tame_speed(v);
         double v2, v3, v4, xn, vn, an;
         bool pw = true;
-        if (__all_sync(kFull, !active || (held && tame_speed(v)))) {
-            const double kv1 = q.sub(q.sub(nr, q.mul(q.mul(k, v), v)), gs);
+        if (__all_sync(kFull, !active || (held && fused))) {
+            const double kv1 = accel(q, v, nr);
             v2 = q.add(v, q.mul(h2, kv1));
-            const double kv2 = q.sub(q.sub(nr, q.mul(q.mul(k, v2), v2)), gs);
+            const double kv2 = accel(q, v2, nr);
             v3 = q.add(v, q.mul(h2, kv2));
-            const double kv3 = q.sub(q.sub(nr, q.mul(q.mul(k, v3), v3)), gs);
+            const double kv3 = accel(q, v3, nr);
             v4 = q.add(v, q.mul(dt, kv3));
-            const double kv4 = q.sub(q.sub(nr, q.mul(q.mul(k, v4), v4)), gs);
+            const double kv4 = accel(q, v4, nr);
             xn = q.combine(x, v, v2, v3, v4);
             vn = q.combine(v, kv1, kv2, kv3, kv4);
             an = lagged ? a : u;  // not read while r is held
         } else {
-            double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
-            if (lagged) {
-                a1 = a;
-                ka1 = q.mul(q.sub(u, a1), it);
-                a2 = q.add(a, q.mul(h2, ka1));
-                ka2 = q.mul(q.sub(u, a2), it);
-                a3 = q.add(a, q.mul(h2, ka2));
-                ka3 = q.mul(q.sub(u, a3), it);
-                a4 = q.add(a, q.mul(dt, ka3));
-                ka4 = q.mul(q.sub(u, a4), it);
-            } else {
-                a1 = a2 = a3 = a4 = u;
-            }
-            // With dt / tau <= 2 the stage demands lie between the first and the
-            // fourth (-a1 smallest when the command is a deceleration, so that
-            // a - u >= 0 from the start, -a4 smallest otherwise): two tests for
-            // the step.
-            // (A piece exists only when dt / tau <= 2, where the lag is stable and
-            // the stage actuator values are finite, so order keys compare them.)
-            const bool dec = M.a_cmd <= 0.0;
-            const long long kfirst = -okey(dec ? a1 : a4), klast = -okey(dec ? a4 : a1);
-            pw = piece >= 0 && kfirst >= klo && klast <= khi && tame_speed(v);
-            const bool lines = __any_sync(kFull, active && pw && (piece == 1 || piece == 2));
-            if (pw) {
-                const double kv1 = accel_piece(q, v, a1, lines);
-                v2 = q.add(v, q.mul(h2, kv1));
-                const double kv2 = accel_piece(q, v2, a2, lines);
-                v3 = q.add(v, q.mul(h2, kv2));
-                const double kv3 = accel_piece(q, v3, a3, lines);
-                v4 = q.add(v, q.mul(dt, kv3));
-                const double kv4 = accel_piece(q, v4, a4, lines);
+            if (__any_sync(kFull, active && fused)) {
+                double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
+                if (lagged) {
+                    a1 = a;
+                    ka1 = q.mul(q.sub(u, a1), it);
+                    a2 = q.add(a, q.mul(h2, ka1));
+                    ka2 = q.mul(q.sub(u, a2), it);
+                    a3 = q.add(a, q.mul(h2, ka2));
+                    ka3 = q.mul(q.sub(u, a3), it);
+                    a4 = q.add(a, q.mul(dt, ka3));
+                    ka4 = q.mul(q.sub(u, a4), it);
+                } else {
+                    a1 = a2 = a3 = a4 = u;
+                }
+                // With dt / tau <= 2 the stage demands lie between the first and
+                // the fourth (-a1 smallest when the command is a deceleration, so
+                // that a - u >= 0 from the start, -a4 smallest otherwise): two
+                // tests for the step.  (The lag is stable and the stage actuator
+                // values are finite, so order keys compare them.)
+                const bool dec = M.a_cmd <= 0.0;
+                const long long kfirst = -okey(dec ? a1 : a4), klast = -okey(dec ? a4 : a1);
+                pw = held || (piece >= 0 && kfirst >= klo && klast <= khi);
+                double kv1, kv2, kv3, kv4;
+                if (__all_sync(kFull, !active || !fused || pw)) {
+                    const bool lines =
+                        __any_sync(kFull, active && !held && (piece == 1 || piece == 2));
+                    kv1 = accel(q, v, r_piece(q, a1, lines));
+                    v2 = q.add(v, q.mul(h2, kv1));
+                    kv2 = accel(q, v2, r_piece(q, a2, lines));
+                    v3 = q.add(v, q.mul(h2, kv2));
+                    kv3 = accel(q, v3, r_piece(q, a3, lines));
+                    v4 = q.add(v, q.mul(dt, kv3));
+                    kv4 = accel(q, v4, r_piece(q, a4, lines));
+                } else {
+                    // some lane crosses a breakpoint: the full minimum for the
+                    // warp (67 operations, where the lane alone would add them
+                    // to the others' 51-59)
+                    kv1 = accel(q, v, r_full(q, a1));
+                    v2 = q.add(v, q.mul(h2, kv1));
+                    kv2 = accel(q, v2, r_full(q, a2));
+                    v3 = q.add(v, q.mul(h2, kv2));
+                    kv3 = accel(q, v3, r_full(q, a3));
+                    v4 = q.add(v, q.mul(dt, kv3));
+                    kv4 = accel(q, v4, r_full(q, a4));
+                }
                 xn = q.combine(x, v, v2, v3, v4);
                 vn = q.combine(v, kv1, kv2, kv3, kv4);
                 an = lagged ? q.combine(a, ka1, ka2, ka3, ka4) : u;
-            } else if (active) {
-                const double kv1 = accel(v, a1);
-                v2 = v + h2 * kv1;
-                const double kv2 = accel(v2, a2);
-                v3 = v + h2 * kv2;
-                const double kv3 = accel(v3, a3);
-                v4 = v + dt * kv3;
-                const double kv4 = accel(v4, a4);
-                xn = x + h6 * (((v + 2.0 * v2) + 2.0 * v3) + v4);
-                vn = v + h6 * (((kv1 + 2.0 * kv2) + 2.0 * kv3) + kv4);
-                an = lagged ? a + h6 * (((ka1 + 2.0 * ka2) + 2.0 * ka3) + ka4) : u;
+                if (held && lagged) an = a;
+            }
+            if (active && !fused) {
+                const Plain p = plain_step<CAP>(x, v, a, u, it, lagged, k, gs, cold(K_F0),
+                                                cold(K_F1), cold(K_R0), cold(K_R1), c, dt, h2, h6);
+                xn = p.x;
+                vn = p.v;
+                an = p.a;
+                pw = false;
             }
         }
         if (!active) return false;
 
+        const bool contact_near = LEAD && !M.lead_moving && ge_pos(xn, d0);  // d0 > 0 and finite here
         if (LEAD && M.lead_moving) {
             const double t0 = from_int(n) * dt, t1 = from_int(n + 1) * dt;
             const double g1 = (d0 + lead_pos(M, t1)) - xn;
@@ -439,24 +552,24 @@ struct Lane64 {
                 const double g0 = (d0 + lead_pos(M, t0)) - x;
                 const double c0 = v - lead_speed(M, t0), c1 = vn - lead_speed(M, t1);
                 const double s = g0 / (g0 - g1);
-                store_out(O, i, AEB_CONTACT, xn, x + s * (xn - x), c0 + s * (c1 - c0),
+                store_out(O, row_of(W, pos, 0.0).o, AEB_CONTACT, xn, x + s * (xn - x), c0 + s * (c1 - c0),
                           ((double)n + s) * dt, n + 1, onset());
                 return true;
             }
-        } else if (LEAD && ge_pos(xn, d0)) {  // d0 > 0 and finite here
+        } else if (contact_near) {
             const double s = (d0 - x) / (xn - x);
-            store_out(O, i, AEB_CONTACT, xn, d0, v + s * (vn - v), ((double)n + s) * dt, n + 1,
+            store_out(O, row_of(W, pos, 0.0).o, AEB_CONTACT, xn, d0, v + s * (vn - v), ((double)n + s) * dt, n + 1,
                       onset());
             return true;
         }
         if (le_zero(vn)) {
             const double s = v / (v - vn);
-            store_out(O, i, AEB_STOP, xn, x + s * (xn - x), 0.0, ((double)n + s) * dt, n + 1,
+            store_out(O, row_of(W, pos, 0.0).o, AEB_STOP, xn, x + s * (xn - x), 0.0, ((double)n + s) * dt, n + 1,
                       onset());
             return true;
         }
         if (n + 1 >= M.n_max) {
-            store_out(O, i, AEB_HORIZON, xn, xn, 0.0, (double)(n + 1) * dt, n + 1, onset());
+            store_out(O, row_of(W, pos, 0.0).o, AEB_HORIZON, xn, xn, 0.0, (double)(n + 1) * dt, n + 1, onset());
             return true;
         }
         x = xn;
@@ -468,6 +581,86 @@ struct Lane64 {
         return false;
     }
 };
+
+// Prepare entries [start, start + cnt) of the processing order (cnt <= 32) into
+// the warp's records, one per lane: the set-up's binary64 divisions run once per
+// ticket at full width instead of once per refilling lane.  Samples that end at
+// once are stored here.
+template <int CAP, bool LEAD, bool TTC>
+__device__ __noinline__ void prepare(const ModelDev &M, const ParamsDev &P, const OutDev &O,
+                                     const WorkDev &W, uint32_t start, int cnt, WarpMem &w)
+{
+    const int j = threadIdx.x & 31;
+    if (j >= cnt) return;
+    const uint32_t pos = position(W, start + (uint32_t)j);
+    const Row rows = row_of(W, pos, M.ttc_thr);
+    const uint64_t i = rows.o;
+    double f[AEB_NFIELDS];
+    load_fields(P, rows.p, f);
+    w.bits[j] = 0;
+    if (!sample_valid(f)) {
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        store_out(O, i, AEB_INVALID, nan, nan, nan, nan, 0, -1);
+        return;
+    }
+    const double k = ((M.rho * f[kCd]) * M.area) / (2.0 * f[kMass]);
+    const bool lagged = f[kTau] > 0.0;
+    const double it = lagged ? 1.0 / f[kTau] : 0.0;
+    const double mu = f[kMu], mh = mu * M.hl;
+    double c, f0 = 0.0, f1 = 0.0, r0 = 0.0, r1 = 0.0;
+    if (CAP == AEB_CAP_LUMPED) {
+        c = (mu * M.g) / (1.0 + mh);
+    } else {
+        c = mu * f[kGc];
+        f0 = (c * M.phi_f) / (1.0 - mh);
+        f1 = (1.0 - M.beta) / (1.0 - mh);
+        r0 = (c * (1.0 - M.phi_f)) / (1.0 + mh);
+        r1 = M.beta / (1.0 + mh);
+    }
+    const int32_t n_delay = steps_to_reach_dev(f[kTdelay], M.dt);
+    const int32_t on = TTC ? -1 : n_delay;
+    if (LEAD && f[kD0] <= 0.0) {
+        store_out(O, i, AEB_CONTACT, 0.0, 0.0, f[kV0], 0.0, 0, on);
+        return;
+    }
+    if (f[kV0] <= 0.0) {
+        store_out(O, i, AEB_STOP, 0.0, 0.0, 0.0, 0.0, 0, on);
+        return;
+    }
+    if (M.n_max == 0) {
+        store_out(O, i, AEB_HORIZON, 0.0, 0.0, 0.0, 0.0, 0, on);
+        return;
+    }
+    // ordered: stage demands in order, and the sample inside the range of the
+    // fused forms (see Ops)
+    const bool ordered = (!lagged || M.dt * it <= 2.0) && M.dt >= 1e-30 && M.dt <= 1.0 &&
+                         fabs(M.a_cmd) <= kTame && k <= 1.0 && fabs(f[kGs]) <= kTame &&
+                         fabs(c) < 1e50 && fabs(f0) < 1e50 && fabs(f1) < 1e50 &&
+                         fabs(r0) < 1e50 && fabs(r1) < 1e50;
+    const bool damped = lagged && M.dt * it <= 1.0 && M.a_cmd < 0.0;
+    w.rec[S_V0][j] = f[kV0];
+    w.rec[S_D0][j] = f[kD0];
+    w.rec[S_GS][j] = f[kGs];
+    w.rec[S_K][j] = k;
+    w.rec[S_IT][j] = it;
+    w.rec[S_KEY][j] = __longlong_as_double((long long)rows.k);
+    w.rec[S_F0][j] = f0;
+    w.rec[S_F1][j] = f1;
+    w.rec[S_R0][j] = r0;
+    w.rec[S_R1][j] = r1;
+    w.rec[S_MG][j] = c;
+    w.rec[S_NOISE][j] = f[kNoise];
+    w.rec[S_THR][j] = rows.thr;
+    w.line[0][j] = (float)f0;
+    w.line[1][j] = (float)f1;
+    w.line[2][j] = (float)r0;
+    w.line[3][j] = (float)r1;
+    w.line[4][j] = (float)c;
+    w.pos[j] = pos;
+    w.delay[j] = n_delay;
+    w.bits[j] = B_RUN | (lagged ? B_LAGGED : 0) | (ordered ? B_ORDERED : 0) |
+                (damped ? B_DAMPED : 0);
+}
 
 #ifndef AEB_FP64_MIN_BLOCKS
 #define AEB_FP64_MIN_BLOCKS 1  // resident blocks per SM the register budget must allow
@@ -493,37 +686,55 @@ k_rollout_fp64(ModelDev M, ParamsDev P, OutDev O, WorkDev W)
     const unsigned t = threadIdx.x ^ (unsigned)(W.n >> 63);
     const Ops q{cst[0][t], cst[1][t], cst[2][t], cst[3][t], cst[4][t], cst[5][t]};
     const unsigned lane = threadIdx.x & 31u;
-    WarpQueue wq;
+    __shared__ WarpMem mem[4];
+    WarpMem &w = mem[threadIdx.x >> 5];
+    Ticket ticket{0, 0, false};
+    int batched = 0;         // entries of the ticket already prepared
+    int used = 0, cnt = 0;   // prepared samples taken, and how many there are
+    bool dry = false;
     Lane64<CAP, LEAD, TTC> L;
+    L.mem = &w;
+    L.lane = (int)lane;
     L.active = false;
-    L.x = L.v = L.a = L.d0 = L.gs = L.noise = L.k = L.it = L.thr = 0.0;
-    L.mg = L.f0 = L.f1 = L.r0 = L.r1 = L.cap = L.pa = L.pb = 0.0;
+    L.x = L.v = L.a = L.d0 = L.gs = L.k = L.it = L.c = L.pa = L.pb = L.nr = 0.0;
     L.klo = L.khi = 0;
-    L.row = 0;
-    L.n = L.n_b = L.n_delay = 0;
+    L.n = L.n_b = L.n_delay = L.n_chk = 0;
+    L.pos = 0;
     L.piece = -1;
     L.trig = L.lagged = L.ordered = L.damped = L.held = false;
-    L.nr = 0.0;
-    L.n_chk = 0;
-    uint64_t oidx = 0;
     unsigned need = kFull;
     for (;;) {
         while (need) {
-            uint32_t pos = 0;
-            const bool got = wq.take(need, W, pos);
-            bool ended = false;
-            if ((need >> lane) & 1u) {
-                L.active = got;
-                if (got) {
-                    const Row rows = row_of(W, pos, M.ttc_thr);
-                    oidx = rows.o;
-                    ended = L.init(M, P, O, rows);
+            if (used >= cnt) {
+                if (!dry && batched >= ticket.count) {
+                    ticket = claim_ticket(W);
+                    batched = 0;
+                    dry = !ticket.ok;
                 }
+                if (dry) {
+                    if ((need >> lane) & 1u) L.active = false;
+                    break;
+                }
+                cnt = min(32, ticket.count - batched);
+                used = 0;
+                __syncwarp();  // every lane has read its record of the previous batch
+                prepare<CAP, LEAD, TTC>(M, P, O, W, ticket.start + (uint32_t)batched, cnt, w);
+                __syncwarp();
+                batched += cnt;
             }
-            need = __ballot_sync(kFull, ended);
+            const int slot = used + __popc(need & lanemask_lt());
+            const bool got = ((need >> lane) & 1u) && slot < cnt;
+            if (got) {
+                L.active = w.bits[slot] & B_RUN;
+                if (L.active) L.take(slot);
+            }
+            const unsigned taken = __ballot_sync(kFull, got);
+            used += __popc(taken);
+            // (a sample that ended at once leaves its lane in need)
+            need = (need & ~taken) | __ballot_sync(kFull, got && !L.active);
         }
         if (!__any_sync(kFull, L.active)) return;
-        need = __ballot_sync(kFull, L.step(M, q, O, oidx));
+        need = __ballot_sync(kFull, L.step(M, q, O, W));
     }
 }
 

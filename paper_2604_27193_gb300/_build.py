@@ -33,7 +33,7 @@ CU_SOURCES = {
     "peaks.cu": ["-fmad=true"],
 }
 CPP_SOURCES = ["capi.cpp", "sampler.cpp", "batch.cpp", "serve.cpp", "sweep.cpp", "stats.cpp"]
-HEADERS = ["aeb_internal.h", "rollout_common.cuh", "host_util.h"]
+HEADERS = ["aeb_internal.h", "rollout_common.cuh", "soft64.h", "host_util.h"]
 
 
 def _sources():

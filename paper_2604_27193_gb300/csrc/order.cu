@@ -305,7 +305,7 @@ cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision 
             k.row0 = w.row0 + first;
             k.n = len;
         }
-        cudaError_t e = cudaMemsetAsync(base, 0, order ? lay.keys : sizeof(unsigned long long), s);
+        cudaError_t e = cudaMemsetAsync(base, 0, order ? lay.keys : 2 * sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
         if (order) {
             auto *hist = reinterpret_cast<uint32_t *>(base + lay.hist);

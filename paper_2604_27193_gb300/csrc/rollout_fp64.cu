@@ -41,9 +41,21 @@
 // held: 32 operations (27 and the position) instead of 51.  order.cu hands a
 // warp samples of one cap class and length, so that its lanes are there
 // together.
+//
+// The unit can be relieved further: its 64 cycles hold 64 issue slots, of which
+// a binary64 multiply or add in integer arithmetic (soft64.h) takes 20-25.  So
+// when a launch fills the GPU, the products and the additions of a small
+// increment to a large value (30 of 51 operations, 18 of 32) run on the integer
+// pipes beside the unit, each the same bits; a step in which one does not apply
+// (a zero, a sum three binades away; ~4 % of a warp's steps) is taken again on
+// the unit.  1e6 rollouts 269 -> 194 ms, 250,007 71 -> 54 ms.  Now bound by
+// latency and issue: per warp step ~24 operations on the unit (60 % busy), 765
+// on the half-rate integer pipe (64 %).  The stages run as a loop: unrolled,
+// the step's 20 KB of code wait on the instruction caches (206 ms).
 #include <climits>
 
 #include "rollout_common.cuh"
+#include "soft64.h"
 
 namespace aeb {
 namespace {
@@ -104,6 +116,20 @@ struct Ops {
     }
 };
 
+// The step constants as factors of software multiplies, and the number of live
+// warps above which a launch uses them (kSoftPerSub per SM sub-partition).  A
+// warp alone is limited by its chain of operations, where a software operation
+// (~100 cycles) is slower than the unit's 64; with four warps per
+// sub-partition the unit and the integer pipes share the work.  Above two,
+// three: 1e5 rollouts 33.6, 29.9 ms (29.2 and 29.9 with either rule; paper
+// preset 46.5, 41.3); all software arithmetic 34.3, none 34.8.
+constexpr unsigned kSoftPerSub = 3;
+struct SoftStep {
+    SoftFactor h2, dt, h6;
+    bool ok;
+    unsigned above;
+};
+
 // Bounds of the states the fused forms are used on: they keep every sum and
 // product of a step below 2^400, so nothing overflows.
 constexpr int kTtcSpan = 256;  // steps one trigger test may cover
@@ -146,7 +172,7 @@ __device__ __forceinline__ double realised(double f0, double f1, double r0, doub
 enum { S_V0, S_D0, S_GS, S_K, S_IT, S_KEY, S_NCOPY,  // KEY: perception-key row, as bits
        S_F0 = S_NCOPY, S_F1, S_R0, S_R1, S_MG, S_NOISE, S_THR, S_N };
 enum { K_F0, K_F1, K_R0, K_R1, K_MG, K_NOISE, K_THR, K_N };  // S_F0 + K_*
-enum { B_RUN = 1, B_LAGGED = 2, B_ORDERED = 4, B_DAMPED = 8 };
+enum { B_RUN = 1, B_LAGGED = 2, B_ORDERED = 4, B_DAMPED = 8, B_SOFT = 16 };
 struct WarpMem {
     double rec[S_N][32];
     double cold[K_N][32];
@@ -286,13 +312,15 @@ struct Lane64 {
     double x, v, a;
     double d0, gs, k, it;
     double c;                     // the constant cap: mu g cos(theta), or the Eq. 5 cap
-    double pa, pb;                // current line pa + pb D (piece 1, 2)
+    double mc;                    // -c (a negation is an operation of the binary64 unit)
+    double npa, pb;               // current line: -r = npa + pb a (piece 1, 2)
     long long klo, khi;           // its demand interval [dlo, dhi] as order keys
     int32_t n, n_b, n_delay;
     uint32_t pos;
     int piece;                    // 0: D, 1, 2: an axle line, 3: the constant cap; -1: none
     bool trig, lagged, ordered;
     bool active;                  // the lane holds a rollout
+    bool soft;                    // k and 1 / tau are factors of software multiplies
     bool damped;                  // dt / tau <= 1: the stage demands approach -a_cmd from below
     bool held;                    // r is the same at every stage until onset, or for good
     double nr;                    // -r while held
@@ -314,7 +342,7 @@ struct Lane64 {
         klo = p.klo;
         khi = p.khi;
         if (CAP != AEB_CAP_LUMPED && piece >= 0) {
-            pa = cold(piece == 2 ? K_R0 : K_F0);
+            npa = -cold(piece == 2 ? K_R0 : K_F0);
             pb = cold(piece == 2 ? K_R1 : K_F1);
         }
     }
@@ -324,15 +352,37 @@ struct Lane64 {
     {
         return q.sub(q.sub(mr, q.mul(q.mul(k, vv), vv)), gs);
     }
+    // The same with the products on the integer pipes.
+    __device__ __forceinline__ double accel_soft(const Ops &q, const SoftFactor &fk, double vv,
+                                                 double mr, uint32_t &range) const
+    {
+        const double t = soft_mul(soft_mul(vv, fk, range), soft_factor(vv), range);
+        return q.sub(q.sub(mr, t), gs);
+    }
     // -r on the current piece (or held): the same value as the full minimum's
-    // for a demand -aa in the piece's interval.  `lines`: some lane of the warp
+    // for a demand -aa in the piece's interval (pa + pb (-aa) and npa + pb aa
+    // round alike).  `lines`: some lane of the warp
     // is on an axle line.
     __device__ __forceinline__ double r_piece(const Ops &q, double aa, bool lines) const
     {
-        double mr = (piece == 0) ? aa : -c;
+        double mr = (piece == 0) ? aa : mc;
         if (CAP != AEB_CAP_LUMPED && lines) {
-            const double rl = q.add(pa, q.mul(pb, -aa));
-            if (piece == 1 || piece == 2) mr = -rl;
+            const double rl = q.add(npa, q.mul(pb, aa));
+            if (piece == 1 || piece == 2) mr = rl;
+        }
+        return held ? nr : mr;
+    }
+    __device__ __forceinline__ double r_piece_soft(const Ops &q, const SoftFactor &fb, double aa,
+                                                   bool lines, uint32_t &range) const
+    {
+        double mr = (piece == 0) ? aa : mc;
+        if (CAP != AEB_CAP_LUMPED && lines) {
+            uint32_t rg = 0;
+            const double rl = q.add(npa, soft_mul(aa, fb, rg));
+            if (piece == 1 || piece == 2) {
+                mr = rl;
+                if (!held) range |= rg;
+            }
         }
         return held ? nr : mr;
     }
@@ -367,7 +417,7 @@ struct Lane64 {
             klo > 0x3f50000000000000ll /* 2^-10 */ && -okey(a) >= klo + 4096 &&
             okey(a) >= okey(M.a_cmd)) {
             held = true;
-            nr = -c;
+            nr = mc;
         } else if (__double_as_longlong(a) == __double_as_longlong(M.a_cmd)) {
             hold_at(a);  // settled: a does not move any more
         }
@@ -388,6 +438,7 @@ struct Lane64 {
         k = w.rec[S_K][slot];
         it = w.rec[S_IT][slot];
         c = w.rec[S_MG][slot];
+        mc = -c;
 #pragma unroll
         for (int f = 0; f < K_N; ++f) mem->cold[f][lane] = w.rec[S_F0 + f][slot];
 #pragma unroll
@@ -399,6 +450,7 @@ struct Lane64 {
         lagged = b & B_LAGGED;
         ordered = b & B_ORDERED;
         damped = b & B_DAMPED;
+        soft = b & B_SOFT;
         trig = !TTC;
         n_b = n_delay;
         x = 0.0;
@@ -457,8 +509,8 @@ struct Lane64 {
 
     // One RK4 step (all lanes of the warp together); true if the lane's rollout
     // ended (stored).
-    __device__ __forceinline__ bool step(const ModelDev &M, const Ops &q, const OutDev &O,
-                                         const WorkDev &W)
+    __device__ __forceinline__ bool step(const ModelDev &M, const Ops &q, const SoftStep &S,
+                                         const OutDev &O, const WorkDev &W, bool use_soft)
     {
         const double dt = q.dt, h2 = q.h2, h6 = q.h6;
         if (TTC && active && !trig && n >= n_chk) test_trigger(M, q);
@@ -472,6 +524,24 @@ struct Lane64 {
         double v2, v3, v4, xn, vn, an;
         bool pw = true;
         if (__all_sync(kFull, !active || (held && fused))) {
+            if (use_soft) {
+                const SoftFactor fk = soft_factor(k);
+                uint32_t rg = soft && S.ok ? 0u : ~0u;
+                double vj = v, kj = accel_soft(q, fk, v, nr, rg), sv = v, sk = kj;
+#pragma unroll 1
+                for (int st = 0; st < 3; ++st) {
+                    const SoftFactor fs = st < 2 ? S.h2 : S.dt;
+                    const double w = st < 2 ? q.two : q.one;
+                    vj = soft_add<false>(v, soft_mul(kj, fs, rg), rg);
+                    kj = accel_soft(q, fk, vj, nr, rg);
+                    sv = __fma_rn(w, vj, sv);
+                    sk = __fma_rn(w, kj, sk);
+                }
+                xn = soft_add<false>(x, soft_mul(sv, S.h6, rg), rg);
+                vn = soft_add<false>(v, soft_mul(sk, S.h6, rg), rg);
+                an = lagged ? a : u;  // not read while r is held
+                if (!__any_sync(kFull, active && soft_bad(rg))) goto stepped;
+            }
             const double kv1 = accel(q, v, nr);
             v2 = q.add(v, q.mul(h2, kv1));
             const double kv2 = accel(q, v2, nr);
@@ -483,6 +553,42 @@ struct Lane64 {
             vn = q.combine(v, kv1, kv2, kv3, kv4);
             an = lagged ? a : u;  // not read while r is held
         } else {
+            if (use_soft && __all_sync(kFull, !active || (fused && soft && lagged && S.ok))) {
+                // (a held lane's actuator is not read: stand-ins keep it in
+                // range; the stages as a loop: the instruction caches bound this)
+                const bool lines = __any_sync(kFull, active && !held && (piece == 1 || piece == 2));
+                const SoftFactor fk = soft_factor(k), fi = soft_factor(it), fb = soft_factor(pb);
+                const double a1 = held ? -1.0 : a, us = held ? -3.0 : u;
+                uint32_t ra = lines && !held && !soft_factor_ok(pb) ? ~0u : 0u, rg = 0;
+                double vj = v, aj = a1, kj = 0.0, kaj = 0.0, sv = v, sk = 0.0, sa = 0.0;
+#pragma unroll 1
+                for (int st = 0; st < 4; ++st) {
+                    if (st > 0) {
+                        const SoftFactor fs = st < 3 ? S.h2 : S.dt;
+                        aj = soft_add<true>(a1, soft_mul(kaj, fs, ra), ra);
+                        vj = soft_add<false>(v, soft_mul(kj, fs, rg), rg);
+                    }
+                    kaj = soft_mul(q.sub(us, aj), fi, ra);
+                    kj = accel_soft(q, fk, vj, r_piece_soft(q, fb, aj, lines, rg), rg);
+                    if (st > 0) {
+                        const double w = st < 3 ? q.two : q.one;
+                        sv = __fma_rn(w, vj, sv);
+                        sk = __fma_rn(w, kj, sk);
+                        sa = __fma_rn(w, kaj, sa);
+                    } else {
+                        sk = kj;
+                        sa = kaj;
+                    }
+                }
+                an = soft_add<true>(a1, soft_mul(sa, S.h6, ra), ra);
+                xn = soft_add<false>(x, soft_mul(sv, S.h6, rg), rg);
+                vn = soft_add<false>(v, soft_mul(sk, S.h6, rg), rg);
+                const bool dec = M.a_cmd <= 0.0;
+                const long long kfirst = -okey(dec ? a1 : aj), klast = -okey(dec ? aj : a1);
+                const bool in = held || (piece >= 0 && kfirst >= klo && klast <= khi && !soft_bad(ra));
+                if (held) an = a;
+                if (__all_sync(kFull, !active || (in && !soft_bad(rg)))) goto stepped;
+            }
             if (__any_sync(kFull, active && fused)) {
                 double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
                 if (lagged) {
@@ -542,6 +648,7 @@ struct Lane64 {
                 pw = false;
             }
         }
+    stepped:
         if (!active) return false;
 
         const bool contact_near = LEAD && !M.lead_moving && ge_pos(xn, d0);  // d0 > 0 and finite here
@@ -659,16 +766,17 @@ __device__ __noinline__ void prepare(const ModelDev &M, const ParamsDev &P, cons
     w.pos[j] = pos;
     w.delay[j] = n_delay;
     w.bits[j] = B_RUN | (lagged ? B_LAGGED : 0) | (ordered ? B_ORDERED : 0) |
-                (damped ? B_DAMPED : 0);
+                (damped ? B_DAMPED : 0) |
+                (soft_factor_ok(k) && (!lagged || soft_factor_ok(it)) ? B_SOFT : 0);
 }
 
 #ifndef AEB_FP64_MIN_BLOCKS
-#define AEB_FP64_MIN_BLOCKS 1  // resident blocks per SM the register budget must allow
+#define AEB_FP64_MIN_BLOCKS 4  // resident blocks per SM the register budget must allow
 #endif
 
 template <int CAP, bool LEAD, bool TTC>
 __global__ void __launch_bounds__(128, AEB_FP64_MIN_BLOCKS)
-k_rollout_fp64(ModelDev M, ParamsDev P, OutDev O, WorkDev W)
+k_rollout_fp64(ModelDev M, SoftStep S, ParamsDev P, OutDev O, WorkDev W)
 {
     // Each lane owns one rollout at a time (Sec. V-A, one thread per sample); a
     // lane whose rollout ends takes the next sample of its warp's ticket, so a
@@ -696,12 +804,19 @@ k_rollout_fp64(ModelDev M, ParamsDev P, OutDev O, WorkDev W)
     L.mem = &w;
     L.lane = (int)lane;
     L.active = false;
-    L.x = L.v = L.a = L.d0 = L.gs = L.k = L.it = L.c = L.pa = L.pb = L.nr = 0.0;
+    L.x = L.v = L.a = L.d0 = L.gs = L.k = L.it = L.c = L.mc = L.npa = L.pb = L.nr = 0.0;
     L.klo = L.khi = 0;
     L.n = L.n_b = L.n_delay = L.n_chk = 0;
     L.pos = 0;
     L.piece = -1;
-    L.trig = L.lagged = L.ordered = L.damped = L.held = false;
+    L.trig = L.lagged = L.ordered = L.damped = L.held = L.soft = false;
+    // Software arithmetic pays while the sub-partitions hold four warps each
+    // (see SoftStep): decided from the launch, and again, once the tickets are
+    // out, from the warps that have ended.  Both ways give the same bits.
+    unsigned long long *ended = W.counter + 1;
+    const unsigned warps = gridDim.x * 4u;
+    bool use_soft = warps > S.above;
+    unsigned steps = 0;
     unsigned need = kFull;
     for (;;) {
         while (need) {
@@ -733,8 +848,13 @@ k_rollout_fp64(ModelDev M, ParamsDev P, OutDev O, WorkDev W)
             // (a sample that ended at once leaves its lane in need)
             need = (need & ~taken) | __ballot_sync(kFull, got && !L.active);
         }
-        if (!__any_sync(kFull, L.active)) return;
-        need = __ballot_sync(kFull, L.step(M, q, O, W));
+        if (!__any_sync(kFull, L.active)) {
+            if (lane == 0) atomicAdd(ended, 1ull);
+            return;
+        }
+        if (use_soft && dry && (++steps & 127u) == 0u)
+            use_soft = warps - (unsigned)*(volatile unsigned long long *)ended > S.above;
+        need = __ballot_sync(kFull, L.step(M, q, S, O, W, use_soft));
     }
 }
 
@@ -757,7 +877,10 @@ cudaError_t launch_t(const ModelDev &m, const ParamsDev &p, const OutDev &o, con
     const uint64_t need_blocks = (tickets_of(w) + 3) / 4;  // one ticket per warp at least
     if (need_blocks < blocks) blocks = need_blocks;
     if (blocks < 1) blocks = 1;
-    kern<<<(unsigned)blocks, 128, 0, s>>>(m, p, o, w);
+    const SoftStep st{soft_factor(m.h2), soft_factor(m.dt), soft_factor(m.h6),
+                      soft_factor_ok(m.h2) && soft_factor_ok(m.dt) && soft_factor_ok(m.h6),
+                      kSoftPerSub * 4u * (unsigned)sms};
+    kern<<<(unsigned)blocks, 128, 0, s>>>(m, st, p, o, w);
     return cudaGetLastError();
 }
 

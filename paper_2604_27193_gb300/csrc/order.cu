@@ -14,10 +14,14 @@
 // loses, drag at a mean speed), 9 ms off the true length in the mean on the
 // single-scenario workload; it decides nothing but the order.  Samples whose
 // braking ends on the constant cap (saturated friction) come first: they last
-// longest, and a warp of them alone needs no actuator once it is there.
+// longest, and a warp of them alone needs no actuator once it is there; among
+// samples of one length (bins of 1/256 of the horizon) those whose r(D) settles
+// early come first, so that a warp's lanes settle together (4 bins of 0.25 s:
+// 1-2 % on most workloads; 512 length bins alone, or 32-128 with 4-16 turn
+// bins: slower).
 //
-// Two kernels before the rollouts: bin every position by (cap class, length),
-// then scatter the positions to their bins' ranges (a counting sort; the
+// Two kernels before the rollouts: bin every position by (cap class, length,
+// turn), then scatter the positions to their bins' ranges (a counting sort; the
 // order inside a bin is free).  72 B read and 8 B written and read per
 // sample.
 #include <algorithm>
@@ -28,9 +32,11 @@
 namespace aeb {
 namespace {
 
-constexpr int kLenBins = 512;                 // over [0, horizon]
+constexpr int kLenBins = 256;                 // over [0, horizon]
+constexpr int kTurnBins = 4;                  // of kTurnBin seconds, the last open
+constexpr float kTurnBin = 0.25f;
 constexpr int kClasses = 3;                   // constant cap, axle line, uncapped demand
-constexpr int kBins = kClasses * kLenBins;
+constexpr int kBins = kClasses * kLenBins * kTurnBins;
 constexpr uint16_t kNoSample = 0xffff;        // a position no tile uses
 constexpr int kOrderThreads = 256;
 constexpr int kScatterItems = 16;             // positions per thread of the scatter
@@ -55,34 +61,37 @@ struct Motion {  // coasting at -a0 until tb, then braking at -b
     }
 };
 
-// Predicted seconds until the rollout ends, and its cap class.
+// Predicted seconds until the rollout ends, its cap class, and the time at
+// which r(D) reaches its last piece.
 __device__ __forceinline__ float predict(const OrderModel &M, const ParamsDev &P, const Row &row,
-                                         int &cls)
+                                         int &cls, float &turn)
 {
     auto f = [&](int j) { return (float)__ldg(P.col[j] + row.p); };
     const float v0 = f(kV0), mu = f(kMu), gs = f(kGs), tau = f(kTau);
     const float mh = mu * M.hl;
-    float r = M.D;
+    float r = M.D, B = 0.0f;  // B: the demand at the last breakpoint below M.D
     cls = 2;
     if (M.lumped) {
         const float c = __fdividef(mu * M.g, 1.0f + mh);
         if (c < r) {
-            r = c;
+            r = B = c;
             cls = 0;
         }
     } else {
         const float mg = mu * M.g;
         const float im = __fdividef(1.0f, 1.0f - mh), ip = __fdividef(1.0f, 1.0f + mh);
-        const float lf = (mg * M.phi_f + (1.0f - M.beta) * M.D) * im;
-        const float lr = (mg * (1.0f - M.phi_f) + M.beta * M.D) * ip;
-        const float line = fminf(lf, lr);
-        if (line < r) {
-            r = line;
+        const float f0 = mg * M.phi_f * im, f1 = (1.0f - M.beta) * im;
+        const float r0 = mg * (1.0f - M.phi_f) * ip, r1 = M.beta * ip;
+        const float lf = f0 + f1 * M.D, lr = r0 + r1 * M.D;
+        if (fminf(lf, lr) < r) {
+            r = fminf(lf, lr);
             cls = 1;
+            B = lf < lr ? __fdividef(f0, 1.0f - f1) : __fdividef(r0, 1.0f - r1);
         }
         if (mg <= r) {
             r = mg;
             cls = 0;
+            B = fmaxf(mg, fmaxf(__fdividef(mg - f0, f1), __fdividef(mg - r0, r1)));
         }
     }
     r = fmaxf(r, 1e-3f);
@@ -104,6 +113,7 @@ __device__ __forceinline__ float predict(const OrderModel &M, const ParamsDev &P
             td += (t > 0.0f) ? fminf(t, M.t_max) : M.t_max;
         }
     }
+    turn = td - tau * __logf(fminf(fmaxf(1.0f - __fdividef(B, M.D), 1e-3f), 1.0f));
     Motion m;
     m.v0 = v0;
     m.a0 = a0;
@@ -150,11 +160,13 @@ k_order_keys(OrderModel M, ParamsDev P, WorkDev W, uint32_t positions,
         uint16_t key = kNoSample;
         if (!W.tiles || p % W.tile < W.tiles[p / W.tile].count) {
             int cls;
-            const float t = predict(M, P, row_of(W, p, (double)M.thr), cls);
+            float turn;
+            const float t = predict(M, P, row_of(W, p, (double)M.thr), cls, turn);
             // longest first; a NaN counts as no time at all
             int len = (t > 0.0f) ? (int)(fminf(t * __fdividef((float)kLenBins, M.t_max), 1e6f)) : 0;
             len = len < kLenBins ? len : kLenBins - 1;
-            key = (uint16_t)(cls * kLenBins + (kLenBins - 1 - len));
+            const int tb = (int)fminf(fmaxf(turn * (1.0f / kTurnBin), 0.0f), kTurnBins - 1.0f);
+            key = (uint16_t)((cls * kLenBins + (kLenBins - 1 - len)) * kTurnBins + tb);
             atomicAdd(&sh[key], 1u);
         }
         keys[p] = key;

@@ -104,11 +104,17 @@ enum { kNoLead = 0, kLeadStationary = 1, kLeadMoving = 2 };
 // What a step takes r + g sin(theta) from: the current piece of r(D), the full
 // minimum, or the constant C (every a_j zero).
 enum { kStepPiece, kStepFullMin, kStepFlat };
-// Steps per trip of a full window.  The kernels' code competes for the
-// instruction caches: both bodies unrolled over the whole window (32) are 1-5 %
-// slower than 16 steps of the piece body and 8 of the flat one (single
-// scenario 1e6 2.44 against 2.40 ms, 2e5 at 0.1 ms 5.3 against 5.0, grid of 216
-// jobs 6.61 against 6.40); 8 or 4 of either are within 1 % of those.
+// Steps per trip of a full window.  Where warps share a sub-partition the
+// kernel's code competes for the instruction caches: both bodies unrolled over
+// the whole window (32) are 1-5 % slower than 16 steps of the piece body and 8
+// of the flat one (single scenario 1e6 2.44 against 2.40 ms, 2e5 at 0.1 ms 5.3
+// against 5.0, grid of 216 jobs 6.61 against 6.40; 8 or 4 of either within 1 %
+// of those; one body for full and short windows, in trips the lanes share: 1-5 %
+// slower).  A launch of at most one warp per sub-partition (LONE) waits for the
+// chain of a step, which the actuator terms are not on, so it keeps the whole
+// window, in the perception kernels too, takes no flat vote and may use more
+// registers (1e4 at 0.1 ms 1.84 against 1.87 ms, TTC 2.05 against 2.15,
+// perception 2.04 against 2.18).
 constexpr int kPieceUnroll = 16, kFlatUnroll = 8;
 static_assert(AEB_FP32_WINDOW % kPieceUnroll == 0 && AEB_FP32_WINDOW % kFlatUnroll == 0,
               "whole trips per window");
@@ -569,18 +575,17 @@ struct Lane32 {
     // own length (the short-window version is a rolled loop, to keep the
     // kernel's code small).
     // FLAT: every lane of the warp is flat(); the actuator terms are C.
-    template <bool FULL, bool FLAT>
+    template <bool FULL, bool FLAT, int UNROLL>
     __device__ __forceinline__ bool step_window(const ModelF32 &F, int len)
     {
         constexpr int KIND = FLAT ? kStepFlat : kStepPiece;
         const float vh0 = vh, vl0 = vl, gh0 = gh, gl0 = gl, e0 = e;
         if (FULL) {
             len = AEB_FP32_WINDOW;
-            constexpr int kTrip = FLAT ? kFlatUnroll : kPieceUnroll;
 #pragma unroll 1
-            for (int t = 0; t < AEB_FP32_WINDOW; t += kTrip) {
+            for (int t = 0; t < AEB_FP32_WINDOW; t += UNROLL) {
 #pragma unroll
-                for (int j = 0; j < kTrip; ++j) step_unchecked<KIND>();
+                for (int j = 0; j < UNROLL; ++j) step_unchecked<KIND>();
             }
         } else {
             // rolled (code size), two steps per trip, then the odd step
@@ -1068,8 +1073,8 @@ __device__ __forceinline__ void flush_batch(const ModelDev &M, const ModelF32 &F
 // One warp walks tiles of kTile samples claimed from a global counter; see the
 // file comment.  No wait on other warps or on the host: the loop ends when the
 // tiles are used up and no lane holds a rollout.
-template <int LEAD, bool TTC, bool PERC>
-__global__ void __launch_bounds__(kThreads, PERC ? 5 : AEB_FP32_MIN_BLOCKS)
+template <int LEAD, bool TTC, bool PERC, bool LONE>
+__global__ void __launch_bounds__(kThreads, LONE ? 2 : PERC ? 5 : AEB_FP32_MIN_BLOCKS)
 k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
 {
     extern __shared__ float smem[];
@@ -1250,17 +1255,20 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
         bool replay = false;
         if (full) {
             // (the perception kernels, whose readings and band code already
-            // fill the instruction cache, run it through the rolled loop: the
-            // unrolled copy costs them more in cache misses than it saves)
+            // fill the instruction cache, run it through the rolled loop unless
+            // their warps are alone: the unrolled copy costs them more in cache
+            // misses than it saves)
             // A warp whose lanes are all flat (order.cu hands a warp samples of
             // one cap class) drops the actuator terms: 16 instructions a step
             // on 16 FMA-pipe slots instead of 18 on 20 (icy roads 2.31 -> 2.03
             // ms per 1e6).  Short windows keep the one body (a second costs
             // what it gains).
-            if (__all_sync(kFull, !active || L.flat())) {
-                if (active) replay = L.template step_window<!PERC, true>(F, len);
+            if (LONE) {
+                if (active) replay = L.template step_window<true, false, AEB_FP32_WINDOW>(F, len);
+            } else if (__all_sync(kFull, !active || L.flat())) {
+                if (active) replay = L.template step_window<!PERC, true, kFlatUnroll>(F, len);
             } else {
-                if (active) replay = L.template step_window<!PERC, false>(F, len);
+                if (active) replay = L.template step_window<!PERC, false, kPieceUnroll>(F, len);
             }
         } else if (PERC && __any_sync(kFull, slot >= 0)) {
             // Band lanes keep their window's states; then the warp tests each
@@ -1312,7 +1320,7 @@ k_rollout_fp32(ModelDev M, ModelF32 F, ParamsDev P, OutDev O, WorkDev W)
                 }
             }
         } else {
-            if (active && len > 0) replay = L.template step_window<false, false>(F, len);
+            if (active && len > 0) replay = L.template step_window<false, false, 2>(F, len);
         }
         // Slow steps (breakpoint crossings, the horizon's last step) after the
         // windows: a window that stopped right before one takes it in the same
@@ -1403,7 +1411,6 @@ template <int LEAD, bool TTC, bool PERC>
 cudaError_t launch_t(const ModelDev &m, const ParamsDev &p, const OutDev &o, const WorkDev &w,
                      const LaunchCfg &cfg, cudaStream_t s)
 {
-    auto kern = k_rollout_fp32<LEAD, TTC, PERC>;
     const int T = (int)w.tile;
     if (T < 32 || T > kTileMax || T % 32) return cudaErrorInvalidValue;
     const size_t smem = smem_per_block<TTC, PERC>(T);
@@ -1412,6 +1419,8 @@ cudaError_t launch_t(const ModelDev &m, const ParamsDev &p, const OutDev &o, con
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    const bool lone = tickets_of(w) <= (uint64_t)sms * 4u;
+    auto kern = lone ? k_rollout_fp32<LEAD, TTC, PERC, true> : k_rollout_fp32<LEAD, TTC, PERC, false>;
     if (smem > 48 * 1024) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

@@ -128,6 +128,15 @@ cudaError_t launch_reduce_jobs(const uint8_t *status, const double *x_ref, const
                                const uint32_t *first, const JobDev *jobs, uint32_t n_jobs,
                                RedPartial *partials, aeb_job_stats *stats, cudaStream_t s);
 
+// Samples 0 .. n_per of every (checked) scenario into consecutive rows.
+void sample_scenarios(const aeb_model &model, const aeb_scenario *scenarios, uint32_t n_scen,
+                      uint64_t n_per, const aeb_params &out);
+
+// Device memory from the library's pool of the current device (capi.cpp), in
+// stream order: nullptr if it cannot be had or the stream is being captured.
+// Freed with cudaFreeAsync.
+void *pool_alloc(size_t bytes, cudaStream_t s);
+
 // Host-side helpers shared by the C-ABI glue.
 int64_t steps_to_reach_host(double t, double dt);
 LaunchCfg launch_cfg(aeb_precision precision);

@@ -47,6 +47,96 @@ void destroy_plan(aeb_batch *b)
     delete b;
 }
 
+// A batched call, checked and laid out: its tables on the host, in one block as
+// they go to the device (jobs, tiles, reduction segments, each job's first
+// segment), then the partials and the rollout's scratch.
+struct Layout {
+    ModelDev md;
+    ParamsDev pd;
+    LaunchCfg cfg;
+    uint32_t T = 0;
+    uint64_t total = 0;  // samples
+    std::vector<JobDev> jobs;
+    std::vector<TileDesc> tiles, red;
+    std::vector<uint32_t> first;
+    size_t o_tiles = 0, o_red = 0, o_first = 0, o_part = 0, o_scratch = 0;
+    size_t scratch = 0;  // bytes
+    size_t bytes() const { return o_scratch + scratch; }
+};
+
+aeb_status lay_out(const char *who, const aeb_model *model, const aeb_job *jobs, uint32_t n_jobs,
+                   const aeb_params *params, aeb_precision precision, const aeb_outputs *out,
+                   const aeb_job_stats *stats, Layout *L)
+{
+    const std::string w = who;
+    if (!jobs || n_jobs == 0 || !stats || !out)
+        return fail(AEB_EINVAL, w + ": NULL argument or no jobs");
+    aeb_status st = check_model(model, &L->md);
+    if (st != AEB_OK) return st;
+    st = check_params(params, &L->pd);
+    if (st != AEB_OK) return st;
+    if (!valid_precision(precision)) return fail(AEB_EINVAL, "unknown precision");
+    if (!out->status || !out->x_ref || !out->v_imp || !out->n_steps)
+        return fail(AEB_EINVAL, w + ": status, x_ref, v_imp and n_steps are required");
+    if (reinterpret_cast<uintptr_t>(stats) % 8 != 0)
+        return fail(AEB_EINVAL, w + ": stats is not 8-byte aligned");
+    L->cfg = launch_cfg(precision);
+    const uint32_t T = L->T = ticket_tile(L->cfg);
+    L->jobs.resize(n_jobs);
+    L->first.resize(n_jobs + 1);
+    for (uint32_t j = 0; j < n_jobs; ++j) {
+        const aeb_job &jb = jobs[j];
+        if (!std::isfinite(jb.ttc_thr)) return fail(AEB_EINVAL, w + ": ttc_thr not finite");
+        L->jobs[j] = JobDev{jb.param_offset, jb.out_offset, jb.n, jb.ttc_thr, jb.key_offset};
+        for (uint64_t f = 0; f < jb.n; f += T)
+            L->tiles.push_back(TileDesc{f, j, (uint32_t)std::min<uint64_t>(T, jb.n - f)});
+        L->first[j] = (uint32_t)L->red.size();
+        for (uint64_t f = 0; f < jb.n; f += kRedSegment)
+            L->red.push_back(TileDesc{f, j, (uint32_t)std::min<uint64_t>(kRedSegment, jb.n - f)});
+        if (L->red.size() > 0xffffffffull) return fail(AEB_EINVAL, w + ": too many reduction segments");
+        L->total += jb.n;
+    }
+    L->first[n_jobs] = (uint32_t)L->red.size();
+    L->o_tiles = a256(sizeof(JobDev) * n_jobs);
+    L->o_red = L->o_tiles + a256(sizeof(TileDesc) * L->tiles.size());
+    L->o_first = L->o_red + a256(sizeof(TileDesc) * L->red.size());
+    L->o_part = L->o_first + a256(sizeof(uint32_t) * L->first.size());
+    L->o_scratch = L->o_part + a256(sizeof(RedPartial) * (L->red.size() + 1));
+    L->scratch = rollout_scratch_bytes((uint64_t)L->tiles.size() * T, precision);
+    return AEB_OK;
+}
+
+// The tables in one block, as they lie on the device.
+std::vector<char> packed(const Layout &L)
+{
+    std::vector<char> b(L.o_part);
+    std::memcpy(b.data(), L.jobs.data(), sizeof(JobDev) * L.jobs.size());
+    if (!L.tiles.empty())
+        std::memcpy(b.data() + L.o_tiles, L.tiles.data(), sizeof(TileDesc) * L.tiles.size());
+    if (!L.red.empty()) std::memcpy(b.data() + L.o_red, L.red.data(), sizeof(TileDesc) * L.red.size());
+    std::memcpy(b.data() + L.o_first, L.first.data(), sizeof(uint32_t) * L.first.size());
+    return b;
+}
+
+// The rollouts and the per-job reduction, with the tables at `base` on the device.
+cudaError_t enqueue(const Layout &L, aeb_precision precision, const aeb_outputs *out,
+                    aeb_job_stats *stats, char *base, cudaStream_t s)
+{
+    const auto *jobs = reinterpret_cast<const JobDev *>(base);
+    const auto *tiles = reinterpret_cast<const TileDesc *>(base + L.o_tiles);
+    const auto *red = reinterpret_cast<const TileDesc *>(base + L.o_red);
+    const auto *first = reinterpret_cast<const uint32_t *>(base + L.o_first);
+    if (!L.tiles.empty()) {
+        const WorkDev w{L.total, L.T, nullptr, tiles, (uint64_t)L.tiles.size(), jobs, 0, 0, nullptr};
+        const cudaError_t e = launch_rollout(L.md, L.pd, precision, out_dev(out), w, L.tiles.data(),
+                                             L.cfg, base + L.o_scratch, L.scratch, s);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_reduce_jobs(out->status, out->x_ref, out->v_imp, out->n_steps, red,
+                              (uint32_t)L.red.size(), first, jobs, (uint32_t)L.jobs.size(),
+                              reinterpret_cast<RedPartial *>(base + L.o_part), stats, s);
+}
+
 }  // namespace
 }  // namespace aeb
 
@@ -60,106 +150,42 @@ extern "C" aeb_status aeb_batch_create(const aeb_model *model, const aeb_job *jo
     clear_error();
     if (!plan) return fail(AEB_EINVAL, "aeb_batch_create: plan is NULL");
     *plan = nullptr;
-    if (!jobs || n_jobs == 0 || !stats || !out)
-        return fail(AEB_EINVAL, "aeb_batch_create: NULL argument or no jobs");
-    ModelDev md;
-    ParamsDev pd;
-    aeb_status st = check_model(model, &md);
+    Layout L;
+    aeb_status st = lay_out("aeb_batch_create", model, jobs, n_jobs, params, precision, out, stats, &L);
     if (st != AEB_OK) return st;
-    st = check_params(params, &pd);
-    if (st != AEB_OK) return st;
-    if (!valid_precision(precision)) return fail(AEB_EINVAL, "unknown precision");
-    if (!out->status || !out->x_ref || !out->v_imp || !out->n_steps)
-        return fail(AEB_EINVAL, "aeb_batch_create: status, x_ref, v_imp and n_steps are required");
-    if (reinterpret_cast<uintptr_t>(stats) % 8 != 0)
-        return fail(AEB_EINVAL, "aeb_batch_create: stats is not 8-byte aligned");
-
-    const LaunchCfg cfg = launch_cfg(precision);
-    const uint32_t T = ticket_tile(cfg);
-    std::vector<JobDev> hj(n_jobs);
-    std::vector<TileDesc> tiles, red;
-    std::vector<uint32_t> first(n_jobs + 1);
-    uint64_t total = 0;
-    for (uint32_t j = 0; j < n_jobs; ++j) {
-        const aeb_job &jb = jobs[j];
-        if (!std::isfinite(jb.ttc_thr)) return fail(AEB_EINVAL, "aeb_batch_create: ttc_thr not finite");
-        hj[j] = JobDev{jb.param_offset, jb.out_offset, jb.n, jb.ttc_thr, jb.key_offset};
-        for (uint64_t f = 0; f < jb.n; f += T)
-            tiles.push_back(TileDesc{f, j, (uint32_t)std::min<uint64_t>(T, jb.n - f)});
-        first[j] = (uint32_t)red.size();
-        for (uint64_t f = 0; f < jb.n; f += kRedSegment)
-            red.push_back(TileDesc{f, j, (uint32_t)std::min<uint64_t>(kRedSegment, jb.n - f)});
-        if (red.size() > 0xffffffffull)
-            return fail(AEB_EINVAL, "aeb_batch_create: too many reduction segments");
-        total += jb.n;
-    }
-    first[n_jobs] = (uint32_t)red.size();
-
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
-    const size_t o_jobs = 0;
-    const size_t o_tiles = o_jobs + a256(sizeof(JobDev) * n_jobs);
-    const size_t o_red = o_tiles + a256(sizeof(TileDesc) * tiles.size());
-    const size_t o_first = o_red + a256(sizeof(TileDesc) * red.size());
-    const size_t o_part = o_first + a256(sizeof(uint32_t) * first.size());
-    const size_t o_scratch = o_part + a256(sizeof(RedPartial) * (red.size() + 1));
-    size_t scratch = rollout_scratch_bytes((uint64_t)tiles.size() * T, precision);
 
     aeb_batch *b = new aeb_batch;
     b->device = dev;
     b->n_jobs = n_jobs;
-    e = cudaMalloc(&b->mem, o_scratch + scratch);
-    if (e == cudaErrorMemoryAllocation && scratch > kCounterBytes) {
+    e = cudaMalloc(&b->mem, L.bytes());
+    if (e == cudaErrorMemoryAllocation && L.scratch > kCounterBytes) {
         cudaGetLastError();
-        scratch = kCounterBytes;  // no room for a processing order: natural order
-        e = cudaMalloc(&b->mem, o_scratch + scratch);
+        L.scratch = kCounterBytes;  // no room for a processing order: natural order
+        e = cudaMalloc(&b->mem, L.bytes());
     }
     if (e != cudaSuccess) {
         delete b;
         return cuda_fail(e, "cudaMalloc(batch plan)");
     }
     char *base = static_cast<char *>(b->mem);
-    auto *djobs = reinterpret_cast<JobDev *>(base + o_jobs);
-    auto *dtiles = reinterpret_cast<TileDesc *>(base + o_tiles);
-    auto *dred = reinterpret_cast<TileDesc *>(base + o_red);
-    auto *dfirst = reinterpret_cast<uint32_t *>(base + o_first);
-    auto *dpart = reinterpret_cast<RedPartial *>(base + o_part);
-    struct {
-        void *d;
-        const void *h;
-        size_t n;
-    } up[] = {{djobs, hj.data(), sizeof(JobDev) * hj.size()},
-              {dtiles, tiles.data(), sizeof(TileDesc) * tiles.size()},
-              {dred, red.data(), sizeof(TileDesc) * red.size()},
-              {dfirst, first.data(), sizeof(uint32_t) * first.size()}};
-    for (auto &u : up) {
-        if (!u.n) continue;
-        e = cudaMemcpy(u.d, u.h, u.n, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) {
-            destroy_plan(b);
-            return cuda_fail(e, "cudaMemcpy(batch tables)");
-        }
+    const std::vector<char> tables = packed(L);
+    e = cudaMemcpy(base, tables.data(), tables.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        destroy_plan(b);
+        return cuda_fail(e, "cudaMemcpy(batch tables)");
     }
-
     cudaStream_t cs = nullptr;
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         destroy_plan(b);
         return cuda_fail(e, "cudaStreamCreate");
     }
-    const OutDev od = out_dev(out);
     e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t le = cudaSuccess;
-        if (!tiles.empty()) {
-            const WorkDev w{total, T, nullptr, dtiles, (uint64_t)tiles.size(), djobs, 0, 0, nullptr};
-            le = launch_rollout(md, pd, precision, od, w, tiles.data(), cfg, base + o_scratch,
-                                scratch, cs);
-        }
-        if (le == cudaSuccess)
-            le = launch_reduce_jobs(out->status, out->x_ref, out->v_imp, out->n_steps, dred,
-                                    (uint32_t)red.size(), dfirst, djobs, n_jobs, dpart, stats, cs);
+        const cudaError_t le = enqueue(L, precision, out, stats, base, cs);
         e = cudaStreamEndCapture(cs, &b->graph);
         if (le != cudaSuccess) e = le;
     }
@@ -193,12 +219,28 @@ extern "C" aeb_status aeb_rollout_batched(const aeb_model *model, const aeb_job 
                                           aeb_precision precision, const aeb_outputs *out,
                                           aeb_job_stats *stats, void *stream)
 {
+    // One shot: no graph, and memory from the library's pool where it has some
+    // (otherwise as a plan).
+    clear_error();
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    Layout L;
+    aeb_status st = lay_out("aeb_batch_create", model, jobs, n_jobs, params, precision, out, stats, &L);
+    if (st != AEB_OK) return st;
+    cudaError_t e = cudaSuccess;
+    if (char *base = static_cast<char *>(pool_alloc(L.bytes(), s))) {
+        const std::vector<char> tables = packed(L);
+        e = cudaMemcpyAsync(base, tables.data(), tables.size(), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = enqueue(L, precision, out, stats, base, s);
+        const cudaError_t f = cudaFreeAsync(base, s), g = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = f != cudaSuccess ? f : g;
+        return e == cudaSuccess ? AEB_OK : cuda_fail(e, "batched rollout");
+    }
     aeb_batch *b = nullptr;
-    aeb_status st = aeb_batch_create(model, jobs, n_jobs, params, precision, out, stats, &b);
+    st = aeb_batch_create(model, jobs, n_jobs, params, precision, out, stats, &b);
     if (st != AEB_OK) return st;
     st = aeb_batch_run(b, stream);
     if (st == AEB_OK) {
-        const cudaError_t e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
+        e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
     }
     destroy_plan(b);

@@ -195,16 +195,17 @@ aeb_status scratch_for(cudaStream_t s, size_t bytes, void **out)
     return AEB_OK;
 }
 
-// Scratch of a rollout's processing order (6 B per sample, 100 MB at most),
-// from a pool of the library's own per device: allocated and freed in stream
-// order, so calls on any streams and threads share it safely, and no more than
-// kPoolKeep bytes stay allocated once the work is done.
+// A pool of the library's own per device, for the scratch of a rollout's
+// processing order (6 B per sample, 100 MB at most) and the buffers of one-shot
+// batched calls and sweeps: allocated and freed in stream order, so calls on any
+// streams and threads share it safely, and no more than kPoolKeep bytes stay
+// allocated once the work is done.
 constexpr uint64_t kPoolKeep = uint64_t(256) << 20;
 std::map<int, cudaMemPool_t> g_pools;
 
-// nullptr if the memory cannot be had (or must not be allocated: a stream being
-// captured); the rollout then runs in natural order.
-void *order_alloc(size_t bytes, cudaStream_t s)
+}  // namespace
+
+void *pool_alloc(size_t bytes, cudaStream_t s)
 {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     int dev = 0;
@@ -241,6 +242,8 @@ void *order_alloc(size_t bytes, cudaStream_t s)
     return nullptr;
 }
 
+namespace {
+
 std::mutex g_cfg_mu;
 LaunchCfg g_cfg[2] = {{128, 0, 256, false}, {128, 0, 32, false}};
 
@@ -253,7 +256,7 @@ aeb_status rollout_impl(const ModelDev &md, const ParamsDev &pd, uint64_t n,
     if (st != AEB_OK) return st;
     const LaunchCfg cfg = launch_cfg(precision);
     const size_t want = rollout_scratch_bytes(n, precision);
-    void *order = want > kCounterBytes ? order_alloc(want, s) : nullptr;
+    void *order = want > kCounterBytes ? pool_alloc(want, s) : nullptr;
     const WorkDev w{n, ticket_tile(cfg), nullptr, nullptr, 0, nullptr, key_base, 0, nullptr};
     cudaError_t e = launch_rollout(md, pd, precision, od, w, nullptr, cfg, order ? order : scratch,
                                    order ? want : kCounterBytes, s);

@@ -5,14 +5,22 @@
 // Counter-based: sample i, quantity q draws from Philox-4x64-10 (Salmon et al.,
 // SC'11) at counter (i, q / 2, 0, 0) under key (seed, scenario_id), words 0-1
 // for even q and 2-3 for odd q.  Any sample range can therefore be produced by
-// any thread, in any order, with the same result; threads split [0, n) into
-// contiguous blocks.  Built with -ffp-contract=off so the binary64 transforms
+// any thread, in any order, with the same result; a call's thread and the
+// library's idle sampling threads take [0, n) in pieces of kGrain samples.  Built with -ffp-contract=off so the binary64 transforms
 // round the same on every host.
+#include <pthread.h>
+
+#include <algorithm>
+#include <atomic>
+#include <chrono>
 #include <cmath>
+#include <condition_variable>
 #include <cstring>
+#include <functional>
+#include <list>
+#include <mutex>
 #include <string>
 #include <thread>
-#include <vector>
 
 #include "aeb_internal.h"
 #include "host_util.h"
@@ -164,6 +172,123 @@ bool dist_ok(const aeb_dist &d)
     return true;
 }
 
+// Samples a piece takes on one thread (~170 ns each): ~45 us, a few times what
+// waking a thread costs.
+constexpr uint64_t kGrain = 256;
+
+// Sampling threads shared by every call of the process.  Starting and joining
+// 16 threads takes ~1 ms, more than sampling 50,000 samples on them; these are
+// started when a call first wants them (one fewer than the host's threads), wait
+// for work and end after a second without any.  The calling thread works too
+// and only waits for pieces a helper has begun, so a call never depends on a
+// helper being there.
+class Workers {
+  public:
+    using Piece = std::function<void(uint64_t, uint64_t)>;
+
+    static Workers &get()
+    {
+        static std::once_flag once;
+        std::call_once(once, [] {
+            instance() = new Workers;  // never destroyed: helpers may outlive static objects
+            // a forked child has none of the parent's threads
+            pthread_atfork(nullptr, nullptr, [] { instance() = new Workers; });
+        });
+        return *instance();
+    }
+
+    // f over [0, n) in pieces, on at most `threads` threads, this one included.
+    void run(uint64_t n, unsigned threads, const Piece &f)
+    {
+        Job job(n, &f, threads > 0 ? threads - 1 : 0);
+        const uint64_t pieces = (n + kGrain - 1) / kGrain;
+        const unsigned helpers =
+            (unsigned)std::min<uint64_t>({job.max_helpers, pieces - 1, max_threads_});
+        if (helpers > 0) {
+            std::lock_guard<std::mutex> lk(mu_);
+            jobs_.push_back(&job);
+            while (idle_ + starting_ < helpers && threads_ < max_threads_) {
+                try {
+                    std::thread([this] { loop(); }).detach();
+                } catch (...) {
+                    break;  // fewer helpers
+                }
+                ++threads_;
+                ++starting_;
+            }
+            work_.notify_all();
+        }
+        job.take();
+        if (helpers > 0) {
+            std::unique_lock<std::mutex> lk(mu_);
+            jobs_.remove(&job);
+            done_.wait(lk, [&] { return job.helpers == 0; });
+        }
+    }
+
+  private:
+    struct Job {
+        const uint64_t n;
+        const Piece *f;
+        const unsigned max_helpers;
+        std::atomic<uint64_t> next{0};
+        unsigned helpers = 0;  // threads inside take(), under the pool's lock
+        Job(uint64_t n_, const Piece *f_, unsigned m) : n(n_), f(f_), max_helpers(m) {}
+        void take()
+        {
+            for (uint64_t lo; (lo = next.fetch_add(kGrain)) < n;)
+                (*f)(lo, std::min(n, lo + kGrain));
+        }
+    };
+
+    static Workers *&instance()
+    {
+        static Workers *w = nullptr;
+        return w;
+    }
+
+    void loop()
+    {
+        std::unique_lock<std::mutex> lk(mu_);
+        --starting_;
+        for (;;) {
+            Job *job = nullptr;
+            for (Job *j : jobs_)
+                if (j->helpers < j->max_helpers && j->next.load() < j->n) {
+                    job = j;
+                    break;
+                }
+            if (!job) {
+                ++idle_;
+                const auto r = work_.wait_for(lk, std::chrono::seconds(1));
+                --idle_;
+                if (r == std::cv_status::timeout && jobs_.empty()) {
+                    --threads_;
+                    return;
+                }
+                continue;
+            }
+            ++job->helpers;
+            lk.unlock();
+            job->take();
+            lk.lock();
+            if (--job->helpers == 0) done_.notify_all();  // the job may be gone after this
+        }
+    }
+
+    std::mutex mu_;
+    std::condition_variable work_, done_;
+    std::list<Job *> jobs_;
+    unsigned threads_ = 0, idle_ = 0, starting_ = 0;
+    const unsigned max_threads_ = std::max(2u, std::thread::hardware_concurrency()) - 1;
+};
+
+unsigned sampling_threads(int32_t n_threads)
+{
+    const unsigned hw = std::thread::hardware_concurrency();
+    return n_threads > 0 ? (unsigned)n_threads : (hw ? hw : 1);
+}
+
 }  // namespace
 }  // namespace aeb
 
@@ -199,34 +324,33 @@ aeb_status sample_impl(const char *who, const aeb_model *model, const aeb_scenar
     for (int j = 0; j < AEB_NFIELDS; ++j)
         if (!cols[j]) return fail(AEB_EINVAL, w + ": NULL output column");
 
-    unsigned hw = std::thread::hardware_concurrency();
-    uint64_t t = n_threads > 0 ? (uint64_t)n_threads : (hw ? hw : 1);
-    const uint64_t min_per_thread = 2048;
-    if (t > (n + min_per_thread - 1) / min_per_thread) t = (n + min_per_thread - 1) / min_per_thread;
-    if (t < 1) t = 1;
     const aeb_scenario sc = *scenario;
     const aeb_params o = *out;
-    if (t == 1) {
-        sample_block(model->g, sc, first, 0, n, o, nominal, weights);
-        return AEB_OK;
-    }
-    std::vector<std::thread> pool;
-    pool.reserve(t);
-    try {
-        for (uint64_t k = 0; k < t; ++k) {
-            const uint64_t lo = n * k / t, hi = n * (k + 1) / t;
-            pool.emplace_back(sample_block, model->g, std::cref(sc), first, lo, hi, std::cref(o),
-                              nominal, weights);
-        }
-    } catch (...) {
-        for (auto &th : pool) th.join();
-        return fail(AEB_ENOMEM, w + ": could not start sampling threads");
-    }
-    for (auto &th : pool) th.join();
+    Workers::get().run(n, sampling_threads(n_threads), [&](uint64_t lo, uint64_t hi) {
+        sample_block(model->g, sc, first, lo, hi, o, nominal, weights);
+    });
     return AEB_OK;
 }
 
 }  // namespace
+
+void sample_scenarios(const aeb_model &model, const aeb_scenario *scenarios, uint32_t n_scen,
+                      uint64_t n_per, const aeb_params &out)
+{
+    const auto piece = [&](uint64_t lo, uint64_t hi) {
+        while (lo < hi) {  // the part of [lo, hi) in one scenario
+            const uint64_t sc = lo / n_per, base = sc * n_per, end = std::min(hi, base + n_per);
+            aeb_params o = out;
+            double **c[AEB_NFIELDS] = {&o.v0, &o.d0, &o.mu, &o.gs, &o.gc,
+                                       &o.mass, &o.cd, &o.tau, &o.t_delay, &o.noise};
+            for (auto p : c) *p += base;
+            sample_block(model.g, scenarios[sc], 0, lo - base, end - base, o, nullptr, nullptr);
+            lo = end;
+        }
+    };
+    Workers::get().run(n_scen * n_per, sampling_threads(0), piece);
+}
+
 }  // namespace aeb
 
 extern "C" aeb_status aeb_sample_params(const aeb_model *model, const aeb_scenario *scenario,

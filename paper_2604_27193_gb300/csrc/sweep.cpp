@@ -1,8 +1,12 @@
 // sweep.cpp -- the TTC-threshold sweep: collision probability with a 95 %
 // Wilson interval at each threshold (aeb_wilson, stats.cpp), pooled over
 // scenarios, from batched launches that share one resident parameter block.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
+#include <new>
+#include <utility>
 #include <vector>
 
 #include "aeb_internal.h"
@@ -34,44 +38,48 @@ extern "C" aeb_status aeb_ttc_sweep(const aeb_model *model, const aeb_scenario *
     uint32_t chunk = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(n_thr, max_rows / P));
     const uint64_t out_rows = (uint64_t)chunk * P;
 
-    std::vector<void *> allocs;
+    // device buffers from the library's pool (kept there, up to its bound), else
+    // their own allocations
+    std::vector<std::pair<void *, bool>> allocs;
     auto cleanup = [&] {
-        for (void *p : allocs) cudaFree(p);
+        for (auto &a : allocs)
+            if (a.second) cudaFreeAsync(a.first, s);
+            else cudaFree(a.first);
     };
     auto dalloc = [&](size_t bytes, void **p) {
-        cudaError_t e = cudaMalloc(p, bytes);
-        if (e == cudaSuccess) allocs.push_back(*p);
-        return e;
+        *p = pool_alloc(bytes, s);
+        const bool pooled = *p != nullptr;
+        const cudaError_t r = pooled ? cudaSuccess : cudaMalloc(p, bytes);
+        if (r == cudaSuccess) allocs.emplace_back(*p, pooled);
+        return r;
     };
-    // parameters: sample on the host (pinned), upload once
-    double *hbuf = nullptr;
-    cudaError_t e = cudaHostAlloc(&hbuf, sizeof(double) * AEB_NFIELDS * P, cudaHostAllocDefault);
-    if (e != cudaSuccess) return cuda_fail(e, "aeb_ttc_sweep: pinned staging");
-    void *dpar = nullptr;
-    e = dalloc(sizeof(double) * AEB_NFIELDS * P, &dpar);
-    if (e != cudaSuccess) {
-        cudaFreeHost(hbuf);
-        return cuda_fail(e, "aeb_ttc_sweep: parameter buffer");
+    for (uint32_t sc = 0; sc < n_scen; ++sc) {  // the scenarios' checks (no samples drawn)
+        aeb_params none;
+        std::memset(&none, 0, sizeof none);
+        st = aeb_sample_params(&m, &scenarios[sc], 0, 0, &none, 0);
+        if (st != AEB_OK) return st;
     }
+    // parameters: sample all scenarios on the host, upload once (from pageable
+    // memory, which the driver copies about as fast as pinned memory here; the
+    // pages would take longer to pin: 6.4 MB 0.3 ms to pin, 0.2 to release)
+    std::unique_ptr<double[]> hbuf(new (std::nothrow) double[AEB_NFIELDS * P]);
+    if (!hbuf) return fail(AEB_ENOMEM, "aeb_ttc_sweep: parameter staging");
+    void *dpar = nullptr;
+    cudaError_t e = dalloc(sizeof(double) * AEB_NFIELDS * P, &dpar);
+    if (e != cudaSuccess) return cuda_fail(e, "aeb_ttc_sweep: parameter buffer");
     aeb_params hp, dp;
     double **hc[AEB_NFIELDS] = {&hp.v0, &hp.d0, &hp.mu, &hp.gs, &hp.gc, &hp.mass, &hp.cd, &hp.tau, &hp.t_delay, &hp.noise};
     double **dc[AEB_NFIELDS] = {&dp.v0, &dp.d0, &dp.mu, &dp.gs, &dp.gc, &dp.mass, &dp.cd, &dp.tau, &dp.t_delay, &dp.noise};
     for (int f = 0; f < AEB_NFIELDS; ++f) {
-        *hc[f] = hbuf + (uint64_t)f * P;
+        *hc[f] = hbuf.get() + (uint64_t)f * P;
         *dc[f] = static_cast<double *>(dpar) + (uint64_t)f * P;
     }
-    for (uint32_t sc = 0; sc < n_scen && st == AEB_OK; ++sc) {
-        aeb_params part;
-        double **pc[AEB_NFIELDS] = {&part.v0, &part.d0, &part.mu, &part.gs, &part.gc, &part.mass, &part.cd, &part.tau, &part.t_delay, &part.noise};
-        for (int f = 0; f < AEB_NFIELDS; ++f) *pc[f] = *hc[f] + (uint64_t)sc * n_per;
-        st = aeb_sample_params(&m, &scenarios[sc], 0, n_per, &part, 0);
-    }
-    if (st == AEB_OK) {
-        e = cudaMemcpyAsync(dpar, hbuf, sizeof(double) * AEB_NFIELDS * P, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) st = cuda_fail(e, "aeb_ttc_sweep: parameter upload");
-    }
-    cudaFreeHost(hbuf);
+    sample_scenarios(m, scenarios, n_scen, n_per, hp);
+    e = cudaMemcpyAsync(dpar, hbuf.get(), sizeof(double) * AEB_NFIELDS * P, cudaMemcpyHostToDevice,
+                        s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) st = cuda_fail(e, "aeb_ttc_sweep: parameter upload");
+    hbuf.reset();
     if (st != AEB_OK) {
         cleanup();
         return st;
@@ -102,8 +110,9 @@ extern "C" aeb_status aeb_ttc_sweep(const aeb_model *model, const aeb_scenario *
         st = aeb_rollout_batched(&m, jobs.data(), (uint32_t)jobs.size(), &dp, precision, &out,
                                  static_cast<aeb_job_stats *>(dstats), stream);
         if (st != AEB_OK) break;
-        e = cudaMemcpy(hstats.data(), dstats, sizeof(aeb_job_stats) * jobs.size(),
-                       cudaMemcpyDeviceToHost);
+        e = cudaMemcpyAsync(hstats.data(), dstats, sizeof(aeb_job_stats) * jobs.size(),
+                            cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) {
             st = cuda_fail(e, "aeb_ttc_sweep: statistics copy");
             break;

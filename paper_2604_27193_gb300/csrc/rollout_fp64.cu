@@ -48,10 +48,14 @@
 // increment to a large value (30 of 51 operations, 18 of 32) run on the integer
 // pipes beside the unit, each the same bits; a step in which one does not apply
 // (a zero, a sum three binades away; ~4 % of a warp's steps) is taken again on
-// the unit.  1e6 rollouts 269 -> 194 ms, 250,007 71 -> 54 ms.  Now bound by
-// latency and issue: per warp step ~24 operations on the unit (60 % busy), 765
-// on the half-rate integer pipe (64 %).  The stages run as a loop: unrolled,
-// the step's 20 KB of code wait on the instruction caches (206 ms).
+// the unit.  1e6 rollouts 262 -> 169 ms, 250,007 69 -> 48 ms.  Bound by latency
+// and issue: per warp step ~24 operations on the unit (60 % busy), 765 on the
+// half-rate integer pipe (64 %).  The stages run as a loop: unrolled, the step's
+// 20 KB of code wait on the instruction caches (+6 %).
+//
+// Steps run in runs (Lane64::run) with no event test inside, each step's state
+// tested while the next is computed: a warp alone took 2,740 cycles for a held
+// step and 4,540 for another, now 2,300 (2,048 on the unit) and 3,850.
 #include <climits>
 
 #include "rollout_common.cuh"
@@ -119,11 +123,11 @@ struct Ops {
 // The step constants as factors of software multiplies, and the number of live
 // warps above which a launch uses them (kSoftPerSub per SM sub-partition).  A
 // warp alone is limited by its chain of operations, where a software operation
-// (~100 cycles) is slower than the unit's 64; with four warps per
-// sub-partition the unit and the integer pipes share the work.  Above two,
-// three: 1e5 rollouts 33.6, 29.9 ms (29.2 and 29.9 with either rule; paper
-// preset 46.5, 41.3); all software arithmetic 34.3, none 34.8.
-constexpr unsigned kSoftPerSub = 3;
+// (~100 cycles) is slower than the unit's 64; from three warps per sub-partition
+// on the unit and the integer pipes share the work.  Above two, three: 45,000
+// rollouts 16.0, 21.4 ms (paper preset 20.6, 27.6; braking lead 14.1, 19.4);
+// at 30,000 and from 65,000 on alike.
+constexpr unsigned kSoftPerSub = 2;
 struct SoftStep {
     SoftFactor h2, dt, h6;
     bool ok;
@@ -133,6 +137,7 @@ struct SoftStep {
 // Bounds of the states the fused forms are used on: they keep every sum and
 // product of a step below 2^400, so nothing overflows.
 constexpr int kTtcSpan = 256;  // steps one trigger test may cover
+constexpr int kRunHeld = 64, kRunPiece = 16;  // steps of a run (a piece's end in a hold is seen after it)
 constexpr double kTame = 1e5;
 __device__ __forceinline__ bool tame_speed(double v)  // 0 < v < ~1e5 (false for a NaN)
 {
@@ -306,6 +311,12 @@ __device__ __noinline__ Plain plain_step(double x, double v, double a, double u,
     p.a = lagged ? a + h6 * (((ka1 + 2.0 * ka2) + 2.0 * ka3) + ka4) : u;
     return p;
 }
+
+// A bool known when compiling, for a generic lambda.
+template <bool B>
+struct Constant {
+    __device__ __forceinline__ constexpr operator bool() const { return B; }
+};
 
 template <int CAP, bool LEAD, bool TTC>
 struct Lane64 {
@@ -507,10 +518,247 @@ struct Lane64 {
         }
     }
 
-    // One RK4 step (all lanes of the warp together); true if the lane's rollout
-    // ended (stored).
-    __device__ __forceinline__ bool step(const ModelDev &M, const Ops &q, const SoftStep &S,
-                                         const OutDev &O, const WorkDev &W, bool use_soft)
+    // The end of the step from (x0, v0) at step n0 to (x1, v1): contact, stop or
+    // the horizon, refined and stored; false if the rollout goes on.
+    __device__ __forceinline__ bool finish(const ModelDev &M, const Ops &q, const OutDev &O,
+                                           const WorkDev &W, double x0, double v0, int32_t n0,
+                                           double x1, double v1) const
+    {
+        const double dt = q.dt;
+        if (LEAD && M.lead_moving) {
+            const double t0 = from_int(n0) * dt, t1 = from_int(n0 + 1) * dt;
+            const double g1 = (d0 + lead_pos(M, t1)) - x1;
+            if (g1 <= 0.0) {
+                const double g0 = (d0 + lead_pos(M, t0)) - x0;
+                const double c0 = v0 - lead_speed(M, t0), c1 = v1 - lead_speed(M, t1);
+                const double s = g0 / (g0 - g1);
+                store_out(O, row_of(W, pos, 0.0).o, AEB_CONTACT, x1, x0 + s * (x1 - x0),
+                          c0 + s * (c1 - c0), ((double)n0 + s) * dt, n0 + 1, onset());
+                return true;
+            }
+        } else if (LEAD && ge_pos(x1, d0)) {  // d0 > 0 and finite here
+            const double s = (d0 - x0) / (x1 - x0);
+            store_out(O, row_of(W, pos, 0.0).o, AEB_CONTACT, x1, d0, v0 + s * (v1 - v0),
+                      ((double)n0 + s) * dt, n0 + 1, onset());
+            return true;
+        }
+        if (le_zero(v1)) {
+            const double s = v0 / (v0 - v1);
+            store_out(O, row_of(W, pos, 0.0).o, AEB_STOP, x1, x0 + s * (x1 - x0), 0.0,
+                      ((double)n0 + s) * dt, n0 + 1, onset());
+            return true;
+        }
+        if (n0 + 1 >= M.n_max) {
+            store_out(O, row_of(W, pos, 0.0).o, AEB_HORIZON, x1, x1, 0.0, (double)(n0 + 1) * dt,
+                      n0 + 1, onset());
+            return true;
+        }
+        return false;
+    }
+
+    // How many steps from here need none of step()'s event tests: before the
+    // horizon's last step, the onset, the next trigger test and, with a moving
+    // lead, before the gap can have closed (the car's acceleration is at most
+    // |g sin(theta)| while its demand is not negative; the lead's travel only
+    // widens the gap).
+    __device__ __forceinline__ int room(const ModelDev &M, const Ops &q) const
+    {
+        if (!active) return kRunHeld;
+        if (!(ordered && tame_speed(v) && (held || piece >= 0))) return 0;
+        int r = min(kRunHeld, (M.n_max - 1) - n);
+        if (TTC && !trig) r = min(r, n_chk - n);
+        else if (n <= n_b) r = min(r, n_b - n);
+        if (LEAD && M.lead_moving && r > 0) {
+            if (!(a <= 0.0 && c >= 0.0 && M.a_cmd <= 0.0 &&
+                  (held ? nr <= 0.0
+                        : piece == 0 || piece == 3 || (npa <= 0.0 && pb >= 0.0))))
+                return 0;
+            const double xl = lead_pos(M, from_int(n) * q.dt);
+            const float g = (float)((d0 + xl) - x) * 0.999f -
+                            1e-5f * (fabsf((float)d0) + fabsf((float)xl) + fabsf((float)x));
+            const float dtf = (float)q.dt;
+            const float W = (float)v + (float)kRunHeld * dtf * fabsf((float)gs);
+            const float steps = __fdividef(g, W * dtf * 1.001f);
+            r = steps >= (float)r ? r : steps > 0.0f ? (int)steps : 0;
+        }
+        return r;
+    }
+
+    // One step with r held, from (x, v).
+    template <bool SOFT>
+    __device__ __forceinline__ void held_step(const Ops &q, const SoftStep &S, const SoftFactor &fk,
+                                              double &xn, double &vn, uint32_t &rg) const
+    {
+        if (SOFT) {
+            double vj = v, kj = accel_soft(q, fk, v, nr, rg), sv = v, sk = kj;
+#pragma unroll 1
+            for (int st = 0; st < 3; ++st) {  // (a loop: the instruction caches bound this)
+                const SoftFactor fs = st < 2 ? S.h2 : S.dt;
+                const double w = st < 2 ? q.two : q.one;
+                vj = soft_add<false>(v, soft_mul(kj, fs, rg), rg);
+                kj = accel_soft(q, fk, vj, nr, rg);
+                sv = __fma_rn(w, vj, sv);
+                sk = __fma_rn(w, kj, sk);
+            }
+            xn = soft_add<false>(x, soft_mul(sv, S.h6, rg), rg);
+            vn = soft_add<false>(v, soft_mul(sk, S.h6, rg), rg);
+        } else {
+            const double kv1 = accel(q, v, nr);
+            const double v2 = q.add(v, q.mul(q.h2, kv1));
+            const double kv2 = accel(q, v2, nr);
+            const double v3 = q.add(v, q.mul(q.h2, kv2));
+            const double kv3 = accel(q, v3, nr);
+            const double v4 = q.add(v, q.mul(q.dt, kv3));
+            const double kv4 = accel(q, v4, nr);
+            xn = q.combine(x, v, v2, v3, v4);
+            vn = q.combine(v, kv1, kv2, kv3, kv4);
+        }
+    }
+
+    // One step inside a piece (or held), from (x, v, a); `in`: the stage demands
+    // lie in the piece's interval.  With dt / tau <= 2 they lie between the first
+    // and the fourth (-a1 smallest when the command is a deceleration, so that
+    // a - u >= 0 from the start, -a4 smallest otherwise): two tests for the step.
+    // (The lag is stable and the stage actuator values are finite, so order keys
+    // compare them.)  A lane that is not held has a lag.
+    template <bool SOFT>
+    __device__ __forceinline__ void piece_step(const ModelDev &M, const Ops &q, const SoftStep &S,
+                                               const SoftFactor &fk, double u, bool lines,
+                                               double &xn, double &vn, double &an, bool &in,
+                                               uint32_t &rg) const
+    {
+        const bool dec = M.a_cmd <= 0.0;
+        if (SOFT) {
+            // (a held lane's actuator is not read: stand-ins keep it in range)
+            const SoftFactor fi = soft_factor(it), fb = soft_factor(pb);
+            const double a1 = held ? -1.0 : a, us = held ? -3.0 : u;
+            uint32_t ra = lines && !held && !soft_factor_ok(pb) ? ~0u : 0u;
+            double vj = v, aj = a1, kj = 0.0, kaj = 0.0, sv = v, sk = 0.0, sa = 0.0;
+#pragma unroll 1
+            for (int st = 0; st < 4; ++st) {
+                if (st > 0) {
+                    const SoftFactor fs = st < 3 ? S.h2 : S.dt;
+                    aj = soft_add<true>(a1, soft_mul(kaj, fs, ra), ra);
+                    vj = soft_add<false>(v, soft_mul(kj, fs, rg), rg);
+                }
+                kaj = soft_mul(q.sub(us, aj), fi, ra);
+                kj = accel_soft(q, fk, vj, r_piece_soft(q, fb, aj, lines, rg), rg);
+                if (st > 0) {
+                    const double w = st < 3 ? q.two : q.one;
+                    sv = __fma_rn(w, vj, sv);
+                    sk = __fma_rn(w, kj, sk);
+                    sa = __fma_rn(w, kaj, sa);
+                } else {
+                    sk = kj;
+                    sa = kaj;
+                }
+            }
+            an = soft_add<true>(a1, soft_mul(sa, S.h6, ra), ra);
+            xn = soft_add<false>(x, soft_mul(sv, S.h6, rg), rg);
+            vn = soft_add<false>(v, soft_mul(sk, S.h6, rg), rg);
+            const long long kfirst = -okey(dec ? a1 : aj), klast = -okey(dec ? aj : a1);
+            in = held || (kfirst >= klo && klast <= khi && !soft_bad(ra));
+        } else {
+            const double ka1 = q.mul(q.sub(u, a), it);
+            const double a2 = q.add(a, q.mul(q.h2, ka1));
+            const double ka2 = q.mul(q.sub(u, a2), it);
+            const double a3 = q.add(a, q.mul(q.h2, ka2));
+            const double ka3 = q.mul(q.sub(u, a3), it);
+            const double a4 = q.add(a, q.mul(q.dt, ka3));
+            const double ka4 = q.mul(q.sub(u, a4), it);
+            const double kv1 = accel(q, v, r_piece(q, a, lines));
+            const double v2 = q.add(v, q.mul(q.h2, kv1));
+            const double kv2 = accel(q, v2, r_piece(q, a2, lines));
+            const double v3 = q.add(v, q.mul(q.h2, kv2));
+            const double kv3 = accel(q, v3, r_piece(q, a3, lines));
+            const double v4 = q.add(v, q.mul(q.dt, kv3));
+            const double kv4 = accel(q, v4, r_piece(q, a4, lines));
+            an = q.combine(a, ka1, ka2, ka3, ka4);
+            xn = q.combine(x, v, v2, v3, v4);
+            vn = q.combine(v, kv1, kv2, kv3, kv4);
+            const long long kfirst = -okey(dec ? a : a4), klast = -okey(dec ? a4 : a);
+            in = held || (kfirst >= klo && klast <= khi);
+        }
+    }
+
+    // Up to R (>= 1, warp-uniform, within room() of every lane) steps with no
+    // event among them; true if the lane's rollout ended (stored).  The state a
+    // step starts from is tested while the step is computed, and a step that
+    // turns out not to exist (a lane had ended) or not to stay in a piece is
+    // dropped: the tests' ~100 dependent integer instructions, which a warp
+    // alone on its sub-partition would wait for, run beside the binary64 unit.
+    // `redo`: the next step is one for step().
+    template <bool SOFT>
+    __device__ __forceinline__ bool run(const ModelDev &M, const Ops &q, const SoftStep &S,
+                                        const OutDev &O, const WorkDev &W, int R, bool &redo)
+    {
+        const bool braking = trig && n >= n_b;
+        const double u = braking ? M.a_cmd : 0.0;
+        const SoftFactor fk = soft_factor(k);
+        double x0 = x, v0 = v;  // the last step's start
+        bool e = false;         // (x, v) ends the rollout, or leaves the range of the fused forms
+        int done = 0;
+        redo = false;
+        auto advance = [&](double xn, double vn) {
+            x0 = x;
+            v0 = v;
+            x = xn;
+            v = vn;
+            ++done;
+            e = active && (!tame_speed(v) || le_zero(v) || (LEAD && !M.lead_moving && ge_pos(x, d0)));
+        };
+        if (__all_sync(kFull, !active || held)) {
+#pragma unroll 1
+            do {
+                double xn, vn;
+                uint32_t rg = 0;
+                held_step<SOFT>(q, S, fk, xn, vn, rg);
+                if (__any_sync(kFull, e)) break;
+                if (SOFT && __any_sync(kFull, active && soft_bad(rg))) {
+                    redo = true;
+                    break;
+                }
+                advance(xn, vn);
+            } while (done < R);
+        } else {
+            R = min(R, kRunPiece);
+            // (on the unit a loop each for warps with and without a lane on an
+            // axle line: a test inside the step cuts it into short blocks, 4480
+            // against 3850 cycles for a warp alone; with software arithmetic one
+            // loop: two wait on the instruction caches, 186 against 169 ms per 1e6)
+            auto loop = [&](auto lines) {
+#pragma unroll 1
+                do {
+                    double xn, vn, an;
+                    bool in;
+                    uint32_t rg = 0;
+                    piece_step<SOFT>(M, q, S, fk, u, lines, xn, vn, an, in, rg);
+                    if (__any_sync(kFull, e)) break;
+                    if (!__all_sync(kFull, !active || (in && !(SOFT && soft_bad(rg))))) {
+                        redo = true;
+                        break;
+                    }
+                    if (!held) a = an;
+                    advance(xn, vn);
+                } while (done < R);
+            };
+            const bool lines = CAP != AEB_CAP_LUMPED &&
+                               __any_sync(kFull, active && !held && (piece == 1 || piece == 2));
+            if (SOFT) loop(lines);
+            else if (lines) loop(Constant<true>{});
+            else loop(Constant<false>{});
+        }
+        if (!active) return false;
+        n += done;
+        if (e && finish(M, q, O, W, x0, v0, n - 1, x, v)) return true;
+        if (braking && !held && done > 0) try_hold(M);
+        return false;
+    }
+
+    // One RK4 step with every event it may meet, on the binary64 unit (all lanes
+    // of the warp together); true if the lane's rollout ended (stored).
+    __device__ __forceinline__ bool step(const ModelDev &M, const Ops &q, const OutDev &O,
+                                         const WorkDev &W)
     {
         const double dt = q.dt, h2 = q.h2, h6 = q.h6;
         if (TTC && active && !trig && n >= n_chk) test_trigger(M, q);
@@ -524,24 +772,6 @@ struct Lane64 {
         double v2, v3, v4, xn, vn, an;
         bool pw = true;
         if (__all_sync(kFull, !active || (held && fused))) {
-            if (use_soft) {
-                const SoftFactor fk = soft_factor(k);
-                uint32_t rg = soft && S.ok ? 0u : ~0u;
-                double vj = v, kj = accel_soft(q, fk, v, nr, rg), sv = v, sk = kj;
-#pragma unroll 1
-                for (int st = 0; st < 3; ++st) {
-                    const SoftFactor fs = st < 2 ? S.h2 : S.dt;
-                    const double w = st < 2 ? q.two : q.one;
-                    vj = soft_add<false>(v, soft_mul(kj, fs, rg), rg);
-                    kj = accel_soft(q, fk, vj, nr, rg);
-                    sv = __fma_rn(w, vj, sv);
-                    sk = __fma_rn(w, kj, sk);
-                }
-                xn = soft_add<false>(x, soft_mul(sv, S.h6, rg), rg);
-                vn = soft_add<false>(v, soft_mul(sk, S.h6, rg), rg);
-                an = lagged ? a : u;  // not read while r is held
-                if (!__any_sync(kFull, active && soft_bad(rg))) goto stepped;
-            }
             const double kv1 = accel(q, v, nr);
             v2 = q.add(v, q.mul(h2, kv1));
             const double kv2 = accel(q, v2, nr);
@@ -553,42 +783,6 @@ struct Lane64 {
             vn = q.combine(v, kv1, kv2, kv3, kv4);
             an = lagged ? a : u;  // not read while r is held
         } else {
-            if (use_soft && __all_sync(kFull, !active || (fused && soft && lagged && S.ok))) {
-                // (a held lane's actuator is not read: stand-ins keep it in
-                // range; the stages as a loop: the instruction caches bound this)
-                const bool lines = __any_sync(kFull, active && !held && (piece == 1 || piece == 2));
-                const SoftFactor fk = soft_factor(k), fi = soft_factor(it), fb = soft_factor(pb);
-                const double a1 = held ? -1.0 : a, us = held ? -3.0 : u;
-                uint32_t ra = lines && !held && !soft_factor_ok(pb) ? ~0u : 0u, rg = 0;
-                double vj = v, aj = a1, kj = 0.0, kaj = 0.0, sv = v, sk = 0.0, sa = 0.0;
-#pragma unroll 1
-                for (int st = 0; st < 4; ++st) {
-                    if (st > 0) {
-                        const SoftFactor fs = st < 3 ? S.h2 : S.dt;
-                        aj = soft_add<true>(a1, soft_mul(kaj, fs, ra), ra);
-                        vj = soft_add<false>(v, soft_mul(kj, fs, rg), rg);
-                    }
-                    kaj = soft_mul(q.sub(us, aj), fi, ra);
-                    kj = accel_soft(q, fk, vj, r_piece_soft(q, fb, aj, lines, rg), rg);
-                    if (st > 0) {
-                        const double w = st < 3 ? q.two : q.one;
-                        sv = __fma_rn(w, vj, sv);
-                        sk = __fma_rn(w, kj, sk);
-                        sa = __fma_rn(w, kaj, sa);
-                    } else {
-                        sk = kj;
-                        sa = kaj;
-                    }
-                }
-                an = soft_add<true>(a1, soft_mul(sa, S.h6, ra), ra);
-                xn = soft_add<false>(x, soft_mul(sv, S.h6, rg), rg);
-                vn = soft_add<false>(v, soft_mul(sk, S.h6, rg), rg);
-                const bool dec = M.a_cmd <= 0.0;
-                const long long kfirst = -okey(dec ? a1 : aj), klast = -okey(dec ? aj : a1);
-                const bool in = held || (piece >= 0 && kfirst >= klo && klast <= khi && !soft_bad(ra));
-                if (held) an = a;
-                if (__all_sync(kFull, !active || (in && !soft_bad(rg)))) goto stepped;
-            }
             if (__any_sync(kFull, active && fused)) {
                 double a1, a2, a3, a4, ka1 = 0.0, ka2 = 0.0, ka3 = 0.0, ka4 = 0.0;
                 if (lagged) {
@@ -603,11 +797,7 @@ struct Lane64 {
                 } else {
                     a1 = a2 = a3 = a4 = u;
                 }
-                // With dt / tau <= 2 the stage demands lie between the first and
-                // the fourth (-a1 smallest when the command is a deceleration, so
-                // that a - u >= 0 from the start, -a4 smallest otherwise): two
-                // tests for the step.  (The lag is stable and the stage actuator
-                // values are finite, so order keys compare them.)
+                // (the stage demands in order, as in piece_step)
                 const bool dec = M.a_cmd <= 0.0;
                 const long long kfirst = -okey(dec ? a1 : a4), klast = -okey(dec ? a4 : a1);
                 pw = held || (piece >= 0 && kfirst >= klo && klast <= khi);
@@ -648,37 +838,8 @@ struct Lane64 {
                 pw = false;
             }
         }
-    stepped:
         if (!active) return false;
-
-        const bool contact_near = LEAD && !M.lead_moving && ge_pos(xn, d0);  // d0 > 0 and finite here
-        if (LEAD && M.lead_moving) {
-            const double t0 = from_int(n) * dt, t1 = from_int(n + 1) * dt;
-            const double g1 = (d0 + lead_pos(M, t1)) - xn;
-            if (g1 <= 0.0) {
-                const double g0 = (d0 + lead_pos(M, t0)) - x;
-                const double c0 = v - lead_speed(M, t0), c1 = vn - lead_speed(M, t1);
-                const double s = g0 / (g0 - g1);
-                store_out(O, row_of(W, pos, 0.0).o, AEB_CONTACT, xn, x + s * (xn - x), c0 + s * (c1 - c0),
-                          ((double)n + s) * dt, n + 1, onset());
-                return true;
-            }
-        } else if (contact_near) {
-            const double s = (d0 - x) / (xn - x);
-            store_out(O, row_of(W, pos, 0.0).o, AEB_CONTACT, xn, d0, v + s * (vn - v), ((double)n + s) * dt, n + 1,
-                      onset());
-            return true;
-        }
-        if (le_zero(vn)) {
-            const double s = v / (v - vn);
-            store_out(O, row_of(W, pos, 0.0).o, AEB_STOP, xn, x + s * (xn - x), 0.0, ((double)n + s) * dt, n + 1,
-                      onset());
-            return true;
-        }
-        if (n + 1 >= M.n_max) {
-            store_out(O, row_of(W, pos, 0.0).o, AEB_HORIZON, xn, xn, 0.0, (double)(n + 1) * dt, n + 1, onset());
-            return true;
-        }
+        if (finish(M, q, O, W, x, v, n, xn, vn)) return true;
         x = xn;
         v = vn;
         a = an;
@@ -810,13 +971,13 @@ k_rollout_fp64(ModelDev M, SoftStep S, ParamsDev P, OutDev O, WorkDev W)
     L.pos = 0;
     L.piece = -1;
     L.trig = L.lagged = L.ordered = L.damped = L.held = L.soft = false;
-    // Software arithmetic pays while the sub-partitions hold four warps each
+    // Software arithmetic pays while the sub-partitions hold enough warps
     // (see SoftStep): decided from the launch, and again, once the tickets are
     // out, from the warps that have ended.  Both ways give the same bits.
     unsigned long long *ended = W.counter + 1;
     const unsigned warps = gridDim.x * 4u;
     bool use_soft = warps > S.above;
-    unsigned steps = 0;
+    unsigned runs = 0;
     unsigned need = kFull;
     for (;;) {
         while (need) {
@@ -852,9 +1013,18 @@ k_rollout_fp64(ModelDev M, SoftStep S, ParamsDev P, OutDev O, WorkDev W)
             if (lane == 0) atomicAdd(ended, 1ull);
             return;
         }
-        if (use_soft && dry && (++steps & 127u) == 0u)
-            use_soft = warps - (unsigned)*(volatile unsigned long long *)ended > S.above;
-        need = __ballot_sync(kFull, L.step(M, q, S, O, W, use_soft));
+        const int R = __reduce_min_sync(kFull, L.room(M, q));
+        need = 0;
+        bool redo = true;
+        if (R > 0) {
+            if (use_soft && dry && (++runs & 3u) == 0u)
+                use_soft = warps - (unsigned)*(volatile unsigned long long *)ended > S.above;
+            const bool soft = use_soft && S.ok && __all_sync(kFull, !L.active || L.soft);
+            const bool over = soft ? L.template run<true>(M, q, S, O, W, R, redo)
+                                   : L.template run<false>(M, q, S, O, W, R, redo);
+            need = __ballot_sync(kFull, over);
+        }
+        if (redo) need = __ballot_sync(kFull, L.step(M, q, O, W));
     }
 }
 

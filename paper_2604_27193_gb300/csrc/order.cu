@@ -39,7 +39,11 @@ constexpr int kClasses = 3;                   // constant cap, axle line, uncapp
 constexpr int kBins = kClasses * kLenBins * kTurnBins;
 constexpr uint16_t kNoSample = 0xffff;        // a position no tile uses
 constexpr int kOrderThreads = 256;
-constexpr int kScatterItems = 16;             // positions per thread of the scatter
+// Positions per thread of the scatter: few in a small launch, which waits for
+// one block's chain (1e5: 13.4 -> 7 us), more where the blocks' scans of the
+// counts add up.
+constexpr int kScatterFew = 4, kScatterMany = 16;
+constexpr uint32_t kScatterSmall = 1u << 19;
 // Positions ordered at a time, and so the bound on the scratch (100 MB).  A
 // longer launch runs in pieces; each piece's tail costs ~0.3 ms of ~40.
 constexpr uint64_t kOrderMax = uint64_t(1) << 24;
@@ -50,6 +54,18 @@ struct OrderModel {
     float D, g, rho_a2, hl, beta, phi_f, thr, lat, t_max, lv0, lb, lts, lxs;
     int lumped, ttc, lead, moving;
 };
+
+// x cut to binary32 on the integer pipe (a conversion instruction runs on the
+// binary64 unit, 64 cycles a warp): 0 below the normal range, the largest value
+// above it.  Good enough for an order.
+__device__ __forceinline__ float cut_f32(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t m = hi & 0x7fffffffu;
+    uint32_t b = ((m - (896u << 20)) << 3) | (lo >> 29);
+    b = m < (897u << 20) ? 0u : m >= (1151u << 20) ? 0x7f7fffffu : b;
+    return __int_as_float((int)(b | (hi & 0x80000000u)));
+}
 
 struct Motion {  // coasting at -a0 until tb, then braking at -b
     float v0, a0, tb, v1, x1, b;
@@ -66,7 +82,7 @@ struct Motion {  // coasting at -a0 until tb, then braking at -b
 __device__ __forceinline__ float predict(const OrderModel &M, const ParamsDev &P, const Row &row,
                                          int &cls, float &turn)
 {
-    auto f = [&](int j) { return (float)__ldg(P.col[j] + row.p); };
+    auto f = [&](int j) { return cut_f32(__ldg(P.col[j] + row.p)); };
     const float v0 = f(kV0), mu = f(kMu), gs = f(kGs), tau = f(kTau);
     const float mh = mu * M.hl;
     float r = M.D, B = 0.0f;  // B: the demand at the last breakpoint below M.D
@@ -105,9 +121,10 @@ __device__ __forceinline__ float predict(const OrderModel &M, const ParamsDev &P
     const float d0 = M.lead ? f(kD0) : 0.0f;
     if (M.ttc) {  // coasting until the measured gap reaches thr times the closing speed
         const float lb = M.moving ? M.lb : 0.0f;
-        const float c0 = v0 - M.lv0, C = f(kD0) + f(kNoise) - (float)row.thr * c0;
+        const float thr = cut_f32(row.thr);
+        const float c0 = v0 - M.lv0, C = f(kD0) + f(kNoise) - thr * c0;
         if (C > 0.0f) {
-            const float A = 0.5f * (lb - a0), B = c0 + (float)row.thr * (lb - a0);
+            const float A = 0.5f * (lb - a0), B = c0 + thr * (lb - a0);
             const float q = B * B + 4.0f * A * C;
             const float t = (q > 0.0f) ? __fdividef(2.0f * C, B + sqrtf(q)) : M.t_max;
             td += (t > 0.0f) ? fminf(t, M.t_max) : M.t_max;
@@ -178,6 +195,7 @@ k_order_keys(OrderModel M, ParamsDev P, WorkDev W, uint32_t positions,
 
 // Pass 2: positions to their bins' ranges.  Each block ranks its positions in
 // shared memory and reserves one range per bin it holds.
+template <int ITEMS>
 __global__ void __launch_bounds__(kOrderThreads)
 k_order_scatter(uint32_t positions, const uint32_t *__restrict__ hist,
                 uint32_t *__restrict__ cursor, const uint16_t *__restrict__ keys,
@@ -210,24 +228,27 @@ k_order_scatter(uint32_t positions, const uint32_t *__restrict__ hist,
         base[t * kPer + j] = run;
         run += own[j];
     }
-    const uint32_t p0 = blockIdx.x * (uint32_t)(kOrderThreads * kScatterItems) + t;
-    uint32_t rank[kScatterItems];
-    uint16_t key[kScatterItems];
+    const uint32_t p0 = blockIdx.x * (uint32_t)(kOrderThreads * ITEMS) + t;
+    uint32_t rank[ITEMS];
+    uint16_t key[ITEMS];
 #pragma unroll
-    for (int i = 0; i < kScatterItems; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
         const uint32_t p = p0 + (uint32_t)i * kOrderThreads;
         key[i] = p < positions ? keys[p] : kNoSample;
         rank[i] = key[i] != kNoSample ? atomicAdd(&cnt[key[i]], 1u) : 0u;
     }
     __syncthreads();
+    uint32_t at[kPer];  // (the reservations in flight together)
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
-        const int b = t + j * kOrderThreads;
-        if (cnt[b]) base[b] += atomicAdd(&cursor[b], cnt[b]);
+        const uint32_t c = cnt[t + j * kOrderThreads];
+        at[j] = c ? atomicAdd(&cursor[t + j * kOrderThreads], c) : 0u;
     }
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) base[t + j * kOrderThreads] += at[j];
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kScatterItems; ++i)
+    for (int i = 0; i < ITEMS; ++i)
         if (key[i] != kNoSample) perm[base[key[i]] + rank[i]] = p0 + (uint32_t)i * kOrderThreads;
 }
 
@@ -329,9 +350,10 @@ cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision 
             k_order_keys<<<kb, kOrderThreads, 0, s>>>(order_model(m), p, k, np, hist, keys);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
-            constexpr uint32_t kChunk = kOrderThreads * kScatterItems;
-            k_order_scatter<<<(np + kChunk - 1) / kChunk, kOrderThreads, 0, s>>>(np, hist, cursor,
-                                                                               keys, perm);
+            const bool few = np <= kScatterSmall;
+            const uint32_t chunk = (uint32_t)kOrderThreads * (few ? kScatterFew : kScatterMany);
+            (few ? k_order_scatter<kScatterFew> : k_order_scatter<kScatterMany>)<<<
+                (np + chunk - 1) / chunk, kOrderThreads, 0, s>>>(np, hist, cursor, keys, perm);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
             k.perm = perm;

@@ -350,7 +350,10 @@ struct Lane32 {
         a3 = bb * cf(L_NP3);
         a4 = bb * cf(L_NP4);
         C = (ab - bb * u) + cf(L_GS);
-        eth = (p4 > 0.0f && B < finf()) ? __fdividef(-u - B, p4) : -finf();
+        // (no threshold: -inf marks a flat lane, NaN any other; both compare alike)
+        const bool flat_now = np1() == 0.0f || (bb == 0.0f && p4 > 0.0f && e >= 0.0f);
+        eth = (p4 > 0.0f && B < finf()) ? __fdividef(-u - B, p4)
+                                        : flat_now ? -finf() : __int_as_float(0x7fc00000);
         // e decays by (1 - mP) per step; a window of K steps stays inside the
         // piece if its last step does: e (1 - mP)^(K-1) >= eth (with margin)
         float ethK = eth;
@@ -435,7 +438,7 @@ struct Lane32 {
         const float s23 = q2 + q3, s123 = s23 + q1;
         vl1 = fmaf(nh6s, fmaf(2.0f, s23, q1 + q4), vl);
         gl1 = fmaf(-ndts, s123, fmaf(-6.0f, v1, gl));
-        en = fmaf(nmP, e, e);
+        en = (KIND == kStepFlat) ? e : fmaf(nmP, e, e);  // (see flat())
     }
 
     // Fold the low words into the high words (Fast2Sum; the pairs stay exact).
@@ -489,12 +492,14 @@ struct Lane32 {
         n = n + 1;
     }
 
-    // Whether r + g sin(theta) is C at every stage whatever e: before onset, on
-    // the constant cap, or with an instantaneous actuator (a_j = +-0).
-    __device__ __forceinline__ bool flat() const
-    {
-        return a1 == 0.0f && a2 == 0.0f && a3 == 0.0f && a4 == 0.0f;
-    }
+    // Whether r + g sin(theta) is C at every stage of every step up to the next
+    // state change, whatever e: before onset (a_j = 0, and e = 0), on the
+    // constant cap for good, or with an instantaneous actuator (a_j = +-0).
+    // set_piece marks these lanes, and no others, by eth = -inf.  A flat window
+    // leaves e as it is: the one later reader, the full minimum of the horizon's
+    // step, takes the constant for every e up to the one at which it became the
+    // minimum (the other lines only rise with the demand).
+    __device__ __forceinline__ bool flat() const { return eth == -finf(); }
 
     // A checked step inside the current piece; true if the rollout ended
     // (contact or stop) in this step, which is then not committed (its

@@ -77,6 +77,28 @@ def test_ordered_rollouts_same_bits_fp64(aeb, kind):
     assert a == b
 
 
+@pytest.mark.parametrize("a_cmd", [-6.0, 1.0])
+@pytest.mark.parametrize("dt,t_max", [(1e-3, 1.2), (5e-3, 3.0), (2e-2, 10.0)])
+def test_fp32_lone_and_full_launches_same_bits(aeb, a_cmd, dt, t_max):
+    """A launch of at most one warp per sub-partition takes no flat windows (and
+    so keeps every lane's actuator state); one that fills the GPU does.  Roads and
+    actuators around the flat condition (saturated, no grip, instantaneous, dt / tau
+    past 1.6), ended by the horizon as well as by stops and contacts."""
+    rng = np.random.default_rng(12)
+    m = ai.replace(ai.single_model(dt), t_max=t_max, a_cmd=a_cmd)
+    n, few = 40_960, 2048
+    p = ai.draw_params(m, ai.scenario_from_means(25.0, 0.05, 0.7, 70.0, 3, 0), n, 9)
+    p["tau"] = rng.choice([0.0, dt / 3, dt / 1.7, dt / 1.5, dt, 0.1, 0.3], n)
+    p["mu"][::29] = 0.0
+    p["mu"][3::31] = 6.0  # mu h / L above 1: a falling line
+    P = _device(p)
+    full, lone = aeb.alloc_outputs(n), aeb.alloc_outputs(few)
+    aeb.aeb_rollout(m, P, n, aeb.FP32_COMP, full)
+    aeb.aeb_rollout(m, {k: v[:few].contiguous() for k, v in P.items()}, few, aeb.FP32_COMP, lone)
+    torch.cuda.synchronize()
+    assert _bits({k: v[:few] for k, v in full.items()}) == _bits(lone)
+
+
 def test_order_in_pieces(aeb):
     """2^24 positions are ordered at a time: a launch of 33 more takes two pieces."""
     n = (1 << 24) + 33

@@ -30,14 +30,14 @@ constexpr int kRedWarps = kRedThreads / 32;
 constexpr int kRedUnroll = 2;    // samples a lane loads at a time (4: 1e7 102 against 98 us)
 
 // floor((x - lo) / w) clamped to [0, NBINS - 1] for the power-of-two width
-// w = 2^-k.  (x - lo) is one binary64 subtraction, as in the definition; the
+// w = 2^-k.  y = x - lo is one binary64 subtraction, as in the definition; the
 // exact scaling by 2^k and the floor are done on its bits with integer
 // instructions, which keeps the binary64 pipe (1/64 rate on GB300) for the
 // sums.  y = m 2^ex with the 53-bit significand m, so floor(y 2^k) is m shifted
 // right by -(ex + k); a normal y with ex + k >= -40 is already >= 2^12.
-__device__ __forceinline__ int bin_index(double x, double lo, int k)
+__device__ __forceinline__ int bin_index(double y, int k)
 {
-    const long long b = __double_as_longlong(x - lo);
+    const long long b = __double_as_longlong(y);
     if (b <= 0) return 0;  // +0, or negative (sign bit set)
     const int e = (int)((b >> 52) & 0x7ff);
     unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
@@ -128,7 +128,7 @@ __device__ __forceinline__ void add_value(Moments &m, double x, double one)
 
 // Queue x of the lanes in `mask` (fill: values waiting); once 32 wait, the warp
 // adds and bins them.
-template <bool HIST>
+template <bool HIST, bool SHIFT>
 __device__ __forceinline__ void push(Queue &q, int &fill, unsigned mask, double x, Moments &m,
                                      double one, unsigned *hist, double lo, int k)
 {
@@ -142,11 +142,11 @@ __device__ __forceinline__ void push(Queue &q, int &fill, unsigned mask, double 
         fill -= 32;
         if (lane < fill) q.v[lane] = z;
         add_value(m, y, one);
-        if (HIST) atomicAdd(&hist[bin_index(y, lo, k)], 1u);
+        if (HIST) atomicAdd(&hist[bin_index(SHIFT ? __fma_rn(lo, -one, y) : y, k)], 1u);
         __syncwarp();
     }
 }
-template <bool HIST>
+template <bool HIST, bool SHIFT>
 __device__ __forceinline__ void drain(const Queue &q, int fill, Moments &m, double one,
                                       unsigned *hist, double lo, int k)
 {
@@ -155,7 +155,7 @@ __device__ __forceinline__ void drain(const Queue &q, int fill, Moments &m, doub
     if (lane < fill) {
         const double y = q.v[lane];
         add_value(m, y, one);
-        if (HIST) atomicAdd(&hist[bin_index(y, lo, k)], 1u);
+        if (HIST) atomicAdd(&hist[bin_index(SHIFT ? __fma_rn(lo, -one, y) : y, k)], 1u);
     }
 }
 
@@ -193,12 +193,15 @@ struct RedShared {
 };
 static_assert(sizeof(RedShared) + 8 * AEB_NBINS <= 96 * 1024, "two blocks per SM");
 
+// SHIFT: an origin of the histograms is not 0 (without one the subtraction, a
+// third binary64 operation per 32 values, is left out: x - 0 is x; 1e7 samples
+// 98 -> 78 us).
 // HIST: accumulate the two histograms and let the last block finish the
 // statistics (the count in stats->n, clear at launch, tells which one that is).
 // With a block table, block b reduces rows [out_offset + first, + count) of job
 // table[b].job (a segment of one job), otherwise rows [b chunk, (b+1) chunk) of
 // [0, n).
-template <bool HIST>
+template <bool HIST, bool SHIFT>
 __global__ void __launch_bounds__(kRedThreads, 2)
 k_reduce_partial(const uint8_t *__restrict__ st, const double *__restrict__ xr,
                  const double *__restrict__ vi, const int32_t *__restrict__ ns, uint64_t n,
@@ -259,12 +262,12 @@ k_reduce_partial(const uint8_t *__restrict__ st, const double *__restrict__ xr,
             n_horizon += __popc(horizon);
             n_invalid += __popc(in & ~(stop | contact | horizon));
             steps += (unsigned long long)(long long)c[u];
-            push<HIST>(sh.q.d[w], fill_d, stop, x[u], md, one, sh_d, h.lo_d, k_d);
-            push<HIST>(sh.q.v[w], fill_v, contact, v[u], mv, one, sh_v, h.lo_v, k_v);
+            push<HIST, SHIFT>(sh.q.d[w], fill_d, stop, x[u], md, one, sh_d, h.lo_d, k_d);
+            push<HIST, SHIFT>(sh.q.v[w], fill_v, contact, v[u], mv, one, sh_v, h.lo_v, k_v);
         }
     }
-    drain<HIST>(sh.q.d[w], fill_d, md, one, sh_d, h.lo_d, k_d);
-    drain<HIST>(sh.q.v[w], fill_v, mv, one, sh_v, h.lo_v, k_v);
+    drain<HIST, SHIFT>(sh.q.d[w], fill_d, md, one, sh_d, h.lo_d, k_d);
+    drain<HIST, SHIFT>(sh.q.v[w], fill_v, mv, one, sh_v, h.lo_v, k_v);
     __syncthreads();  // the queues' memory is used anew
     const long long word[kWords - 4] = {
         (long long)steps, __double_as_longlong(md.sum), __double_as_longlong(md.sumsq),
@@ -352,13 +355,13 @@ cudaError_t launch_reduce(const uint8_t *status, const double *x_ref, const doub
     const int g = reduce_blocks_for(n);
     const uint64_t chunk = (n + (uint64_t)g - 1) / (uint64_t)g;
     constexpr int kBytes = (int)(sizeof(RedShared) + 2 * sizeof(unsigned) * AEB_NBINS);
-    cudaError_t e = cudaFuncSetAttribute(k_reduce_partial<true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+    auto kern = (h.lo_d != 0.0 || h.lo_v != 0.0) ? k_reduce_partial<true, true>
+                                                 : k_reduce_partial<true, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(stats, 0, sizeof(aeb_stats), s);
     if (e != cudaSuccess) return e;
-    k_reduce_partial<true><<<g, kRedThreads, kBytes, s>>>(status, x_ref, v_imp, n_steps, n, chunk,
-                                                          nullptr, nullptr, h, -std::ilogb(h.w_d),
-                                                          -std::ilogb(h.w_v), partials, stats);
+    kern<<<g, kRedThreads, kBytes, s>>>(status, x_ref, v_imp, n_steps, n, chunk, nullptr, nullptr, h,
+                                        -std::ilogb(h.w_d), -std::ilogb(h.w_v), partials, stats);
     return cudaGetLastError();
 }
 
@@ -368,7 +371,7 @@ cudaError_t launch_reduce_jobs(const uint8_t *status, const double *x_ref, const
                                RedPartial *partials, aeb_job_stats *stats, cudaStream_t s)
 {
     if (n_blocks > 0) {
-        k_reduce_partial<false><<<n_blocks, kRedThreads, sizeof(RedShared), s>>>(
+        k_reduce_partial<false, false><<<n_blocks, kRedThreads, sizeof(RedShared), s>>>(
             status, x_ref, v_imp, n_steps, 0, 0, blocks, jobs, aeb_hist_spec{}, 0, 0, partials,
             nullptr);
         const cudaError_t e = cudaGetLastError();

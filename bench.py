@@ -54,12 +54,13 @@ SMS, FP32_LANES_PER_SM, SM_MAX_MHZ = 152, 128, 2070.0
 FP32_PEAK_TFLOPS = SMS * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12  # 80.5
 FP64_PEAK_TFLOPS = 1.25  # GB300 dense FP64, nominal
 # DRAM bytes per sample of the FP32 rollout kernel, from one ncu capture at
-# N = 2e6 (199.7 MB per launch); traffic grows in proportion to the samples.
-FP32_TRAFFIC_BYTES_PER_SAMPLE = 199.657728e6 / 2e6
+# N = 2e6 (2,281 MB per launch: 80 B columns gathered and 21 B scattered 1-8 B at a
+# time in processing order); traffic grows in proportion to the samples.
+FP32_TRAFFIC_BYTES_PER_SAMPLE = 2281.113088e6 / 2e6
 # thread instructions the FP32 kernel executes per RK4 lane-step on this
 # workload (ncu smsp__inst_executed x thread_inst_executed_per_inst_executed at
 # N = 2e6, same profile); the issue-slot view of the roofline
-FP32_THREAD_INST_PER_STEP = 22.46
+FP32_THREAD_INST_PER_STEP = 20.61
 FP32_ISSUE_PEAK = SMS * FP32_LANES_PER_SM * SM_MAX_MHZ * 1e6  # lane-instructions/s
 
 
@@ -761,8 +762,9 @@ def main():
                 "steps": args.fp64_steps, "warmup": 1, "dtype": "f64",
                 "achieved_tflops": steps_per_launch * FLOPS_PER_STEP / (ms64 / 1e3) / 1e12,
                 "peak_tflops_nominal": FP64_PEAK_TFLOPS,
-                "note": "no fused multiply-add on this path: its bound is the binary64 "
-                        "add/multiply rate (measured_pipe_peaks.fp64_add_tops)",
+                "note": "bit-identical to the plain definition (multiply and add rounded "
+                        "apart); operations shared between the binary64 unit and the "
+                        "integer pipes, which bound it together",
                 "fp32_error": err}
 
     # the same, from the seed: host sampling (all host threads) inside the
@@ -836,7 +838,8 @@ def main():
                      "launch_ms": roll_ms,
                      "note": "flops counted from the 73-op binary64 definition of a step; the "
                              "kernel runs 18 binary32 instructions per step (12 FFMA, 2 paired "
-                             "FFMA2, 4 FADD), so frac may exceed 1 without skipped work; "
+                             "FFMA2, 4 FADD; 15 where r(D) is constant), so frac may exceed 1 "
+                             "without skipped work; "
                              "issue.frac is the headroom measure",
                      "issue": {"thread_inst_per_step": FP32_THREAD_INST_PER_STEP,
                                "achieved": steps_per_launch * FP32_THREAD_INST_PER_STEP

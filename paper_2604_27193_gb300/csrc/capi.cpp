@@ -289,7 +289,7 @@ aeb_status reduce_impl(const aeb_outputs *out, uint64_t n, const aeb_hist_spec &
 // so the arithmetic starts after a short upload; each later one is kEvalGrow
 // times the one before.  A chunk's copy must end before the previous chunk's
 // rollouts do: an upload moves 80 B per sample (~1.3 ns per sample at the
-// pinned-host copy rate measured on GB300) against ~2.7 ns per sample of
+// pinned-host copy rate measured on GB300) against ~2.3 ns per sample of
 // FP32 rollout, so a chunk may be at most about twice the one before (six
 // times left the GPU waiting for the last chunk's copy).  The host-to-device
 // copy rate differs between machines (60-200 GB/s measured on GB300 machines), so

@@ -6,7 +6,7 @@
 // callers cannot allow that: a real-time control loop whose rules forbid any
 // allocation after start-up, or a process whose device memory is already
 // handed out in full to another allocator, so that a late cudaMalloc may fail.
-// aeb_reduce_noalloc runs the same two kernels with the partials placed in a
+// aeb_reduce_noalloc runs the same kernel with the partials placed in a
 // fixed array compiled into this library instead; it allocates nothing.
 //
 // The array lives in every GPU that loads the library, for the life of the
@@ -24,8 +24,8 @@
 namespace aeb {
 namespace {
 
-// aeb_reduce splits n samples over ceil(n / 8192) blocks (at most 1024); the
-// static array holds 256 partials (26.6 KB), so n is limited to 256 * 8192.
+// Up to 256 * 8192 samples aeb_reduce runs at most 256 blocks (reduce_blocks_for),
+// one partial each; the static array holds 256 (26.6 KB).
 constexpr int kNoAllocPartials = 256;
 static_assert((uint64_t)kNoAllocPartials * 8192 == AEB_REDUCE_NOALLOC_MAX_N,
               "limit in aeb.h must match the static scratch");

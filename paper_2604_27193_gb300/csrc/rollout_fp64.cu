@@ -49,8 +49,8 @@
 // pipes beside the unit, each the same bits; a step in which one does not apply
 // (a zero, a sum three binades away; ~4 % of a warp's steps) is taken again on
 // the unit.  1e6 rollouts 262 -> 169 ms, 250,007 69 -> 48 ms.  Bound by latency
-// and issue: per warp step ~24 operations on the unit (60 % busy), 765 on the
-// half-rate integer pipe (64 %).  The stages run as a loop: unrolled, the step's
+// and issue: per warp step ~24 operations on the unit (75 % busy), ~670 on the
+// half-rate integer pipe (65 %).  The stages run as a loop: unrolled, the step's
 // 20 KB of code wait on the instruction caches (+6 %).
 //
 // Steps run in runs (Lane64::run) with no event test inside, each step's state

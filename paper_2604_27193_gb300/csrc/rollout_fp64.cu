@@ -126,7 +126,9 @@ struct Ops {
 // (~100 cycles) is slower than the unit's 64; from three warps per sub-partition
 // on the unit and the integer pipes share the work.  Above two, three: 45,000
 // rollouts 16.0, 21.4 ms (paper preset 20.6, 27.6; braking lead 14.1, 19.4);
-// at 30,000 and from 65,000 on alike.
+// at 30,000 and from 65,000 on alike.  (A warp alone with only the position's last
+// product and sum in software: 11.35 -> 11.5 ms at 1e4, so its chain is the limit,
+// not the unit's rate.)
 constexpr unsigned kSoftPerSub = 2;
 struct SoftStep {
     SoftFactor h2, dt, h6;

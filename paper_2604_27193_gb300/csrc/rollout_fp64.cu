@@ -1019,8 +1019,13 @@ k_rollout_fp64(ModelDev M, SoftStep S, ParamsDev P, OutDev O, WorkDev W)
         need = 0;
         bool redo = true;
         if (R > 0) {
-            if (use_soft && dry && (++runs & 3u) == 0u)
-                use_soft = warps - (unsigned)*(volatile unsigned long long *)ended > S.above;
+            if (use_soft && dry && (++runs & 3u) == 0u) {
+                // (one reading for the warp: the lanes must agree on the way they
+                // take, which has full-warp votes of its own)
+                unsigned gone = 0;
+                if (lane == 0) gone = (unsigned)*(volatile unsigned long long *)ended;
+                use_soft = warps - __shfl_sync(kFull, gone, 0) > S.above;
+            }
             const bool soft = use_soft && S.ok && __all_sync(kFull, !L.active || L.soft);
             const bool over = soft ? L.template run<true>(M, q, S, O, W, R, redo)
                                    : L.template run<false>(M, q, S, O, W, R, redo);

@@ -478,9 +478,12 @@ struct Lane64 {
     // that does not fire also bounds the steps that cannot (n_chk): while r is
     // held the car's acceleration is at most acc = max(0, -r - g sin(theta)),
     // so over kTtcSpan steps its speed stays below W = v + kTtcSpan dt acc and
-    // the margin (gap + noise) - thr c falls by at most dt (W + |thr| (acc + b_L))
-    // per step (a braking lead's travel only widens the gap; its speed falls by
-    // dt b_L); a reading's noise is at most 3 perc_sigma.
+    // the margin (gap + noise) - thr c falls by at most dt (W + |thr| rate) per
+    // step (a braking lead's travel only widens the gap).  rate bounds the
+    // closing speed's change towards the trigger: for thr >= 0 its rise, acc and
+    // the lead's b_L; for thr < 0 its fall, r + g sin(theta) and the drag at W,
+    // as long as one step of that keeps every stage speed within [-W, W].  A
+    // reading's noise is at most 3 perc_sigma.
     __device__ __forceinline__ void test_trigger(const ModelDev &M, const Ops &q)
     {
         double gap_meas, closing;
@@ -510,13 +513,17 @@ struct Lane64 {
             long long nb = ((long long)n + M.perc_lat) + n_delay;
             n_b = nb > INT_MAX ? INT_MAX : (int32_t)nb;
         } else if (held && margin > 0.0f && tame_speed(v)) {
-            const float dtf = (float)q.dt, acc = fmaxf(0.0f, (float)(nr - gs));
+            const float dtf = (float)q.dt, net = (float)(nr - gs), acc = fmaxf(0.0f, net);
             const float W = (float)v + (float)kTtcSpan * dtf * acc;
-            const float fall = dtf * (W + fabsf((float)thr) * (acc + (float)M.lead_decel)) * 1.001f;
+            const bool rising = __double2hiint(thr) >= 0;  // (the sign: -0 has no term)
+            const float rate = rising ? acc + (float)M.lead_decel
+                                      : fmaxf(0.0f, -net) + (float)k * W * W;
+            const float fall = dtf * (W + fabsf((float)thr) * rate) * 1.001f;
             // margin's own rounding: a few binary32 ulps of what it was formed from
             const float m = margin * 0.999f - 1e-5f * (fabsf((float)gap_meas) + fabsf((float)limit));
             const float steps = __fdividef(m, fall);
-            if (steps > 1.0f) n_chk = n + (steps < (float)kTtcSpan ? (int)steps : kTtcSpan);
+            if (steps > 1.0f && (rising || dtf * rate * 1.001f <= W))
+                n_chk = n + (steps < (float)kTtcSpan ? (int)steps : kTtcSpan);
         }
     }
 

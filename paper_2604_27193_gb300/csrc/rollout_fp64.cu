@@ -436,6 +436,11 @@ struct Lane64 {
         }
     }
 
+    // Whether k is negative (of the model's constants only finiteness is asked:
+    // an air density or area may be): then the car's speed has no bound over a
+    // span of steps, so that every step tests the trigger and a moving lead.
+    __device__ __forceinline__ bool driven() const { return __double2hiint(k) < 0; }
+
     __device__ __forceinline__ int32_t onset() const
     {
         return TTC ? (trig ? n_b : -1) : n_delay;
@@ -483,7 +488,8 @@ struct Lane64 {
     // closing speed's change towards the trigger: for thr >= 0 its rise, acc and
     // the lead's b_L; for thr < 0 its fall, r + g sin(theta) and the drag at W,
     // as long as one step of that keeps every stage speed within [-W, W].  A
-    // reading's noise is at most 3 perc_sigma.
+    // reading's noise is at most 3 perc_sigma.  (None of this holds for a drag
+    // that drives the car, see driven().)
     __device__ __forceinline__ void test_trigger(const ModelDev &M, const Ops &q)
     {
         double gap_meas, closing;
@@ -512,7 +518,7 @@ struct Lane64 {
             trig = true;
             long long nb = ((long long)n + M.perc_lat) + n_delay;
             n_b = nb > INT_MAX ? INT_MAX : (int32_t)nb;
-        } else if (held && margin > 0.0f && tame_speed(v)) {
+        } else if (held && margin > 0.0f && tame_speed(v) && !driven()) {
             const float dtf = (float)q.dt, net = (float)(nr - gs), acc = fmaxf(0.0f, net);
             const float W = (float)v + (float)kTtcSpan * dtf * acc;
             const bool rising = __double2hiint(thr) >= 0;  // (the sign: -0 has no term)
@@ -578,7 +584,7 @@ struct Lane64 {
         if (TTC && !trig) r = min(r, n_chk - n);
         else if (n <= n_b) r = min(r, n_b - n);
         if (LEAD && M.lead_moving && r > 0) {
-            if (!(a <= 0.0 && c >= 0.0 && M.a_cmd <= 0.0 &&
+            if (!(a <= 0.0 && c >= 0.0 && M.a_cmd <= 0.0 && !driven() &&
                   (held ? nr <= 0.0
                         : piece == 0 || piece == 3 || (npa <= 0.0 && pb >= 0.0))))
                 return 0;

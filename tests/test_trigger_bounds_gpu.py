@@ -1,6 +1,8 @@
-"""Trigger tests that the kernels skip may never hide a trigger, also where the margin
-(gap + noise) - thr (v - v_L) falls because the car slows (a negative threshold:
-uphill, drag).  Most samples of every model trigger; binary64 gives the oracle's bits."""
+"""Trigger tests that the kernels skip may never hide a trigger, and steps that run
+without a contact test may never hide a contact, also where the margin (gap + noise)
+- thr (v - v_L) falls because the car slows (a negative threshold: uphill, drag) or
+because drag drives it (a negative air density).  Most samples of every model trigger;
+binary64 gives the oracle's bits."""
 import numpy as np
 import pytest
 
@@ -41,6 +43,12 @@ CASES = {
     "-2 s readings": (_free(-2.0, perc_sigma=1.0, perc_drop=0.2, perc_latency=0.05,
                             perc_seed=5), 0.0, 25.0),
 }
+DRIVEN = {
+    "driven 2 s": (_free(2.0, rho=-20.0), 0.0, 20.0),
+    "driven -2 s": (_free(-2.0, rho=-20.0), 0.0, 20.0),
+    "driven moving lead": (_lead(2.0, 8.0, 0.0, rho=-20.0), 0.0, 20.0),
+    "driven braking lead": (ai.replace(ai.lead_braking_model(dt=2e-3), rho=-20.0), 0.0, 20.0),
+}
 
 
 def _params(case, seed):
@@ -55,9 +63,9 @@ def _params(case, seed):
 
 
 @pytest.mark.parametrize("copies", [1, 45])  # 54,000 rollouts: software arithmetic too
-@pytest.mark.parametrize("kind", list(CASES))
+@pytest.mark.parametrize("kind", list(CASES) + list(DRIVEN))
 def test_fp64_triggers_as_the_oracle(aeb, oracle_mod, kind, copies):
-    case = CASES[kind]
+    case = {**CASES, **DRIVEN}[kind]
     m = case[0]
     if m.perc_sigma > 0 and copies > 1:
         pytest.skip("a copy's readings are keyed by its own row")

@@ -658,18 +658,6 @@ struct Lane32 {
         return ended;
     }
 
-    // TTC trigger (while not yet triggered): (g + noise) - thr v <= 0, with the
-    // exact rounding error of thr * vh; braking starts n_delay steps later.
-    // Returns how many steps (1 .. kTtcSpan; whole windows from K up) may run
-    // before the next test:
-    // before the trigger the car coasts, the stage accelerations are
-    // q = w^2 + C >= C, so over the span the scaled speed stays below
-    // W = w + kTtcSpan s dt max(0, -C)
-    // and the margin falls by at most 6 W + thr' s dt max(0, -C) per step
-    // (the gap by the stage-speed sum, the speed term by the speed gain); the
-    // first L - 1 steps after this one cannot trigger while (L - 1) times that
-    // bound stays below the margin.  With a moving lead the margin is
-    // (g + noise) - thr (v - v_L).
     // The trigger margin (g + noise) - thr v at the current state, scaled by
     // sigma, with the exact rounding error of thr * vh; a moving lead adds its
     // travel to the gap and takes its speed off the closing speed.
@@ -749,19 +737,27 @@ struct Lane32 {
     // Before the trigger the car coasts, the stage accelerations are
     // q = w^2 + C >= C, so over the span the scaled speed stays below
     // W = w + kTtcSpan s dt max(0, -C)
-    // and the margin falls by at most 6 W + thr' s dt max(0, -C) per step
-    // (the gap by the stage-speed sum, the speed term by the speed gain); the
-    // first L - 1 steps after this one cannot trigger while (L - 1) times that
-    // bound stays below the margin.  With a moving lead the margin is
-    // (g + noise) - thr (v - v_L).
+    // and the margin falls by at most 6 W + |thr'| s dt rate per step (the gap
+    // by the stage-speed sum, the speed term by the closing speed's change
+    // towards the trigger); the first L - 1 steps after this one cannot trigger
+    // while (L - 1) times that bound stays below the margin.  With a moving lead
+    // the margin is (g + noise) - thr (v - v_L).  For thr >= 0 the rate is the
+    // closing speed's rise: max(0, -C), and a braking lead's b_L more (its
+    // travel only widens the gap).  For thr < 0 it is its fall, at most
+    // W^2 + max(0, C) while every stage speed stays within [-W, W], which holds
+    // as long as one step of it takes off no more than W; beyond that no step is
+    // skipped.
     __device__ __forceinline__ int ttc_bound(const ModelF32 &F, float m) const
     {
         const float thr_h = cf(L_THRH);
         const float sdt = -ndts, acc = fmaxf(0.0f, -C);
         const float W = fmaf((float)kTtcSpan * sdt, acc, vh + vl);  // speed bound over the span
-        // (a braking lead's speed term falls by thr' s dt b_L per step more;
-        // its travel only widens the gap)
-        const float d = fmaf(6.0f, W, thr_h * sdt * (acc + F.lb)) * 1.001f;
+        float rate = acc + F.lb;
+        if (thr_h < 0.0f) {
+            rate = fmaf(W, W, fmaxf(0.0f, C));
+            if (!(sdt * rate * 1.001f <= W)) rate = finf();  // (then r is 0)
+        }
+        const float d = fmaf(6.0f, W, fabsf(thr_h) * sdt * rate) * 1.001f;
         // a reading's noise is at most 3 perc_sigma: only a margin beyond that
         // rules a trigger out whatever the readings of the skipped steps
         const float mw = PERC ? fmaf(-3.0f * F.psig, cf(L_SIGMA), m) : m;

@@ -2,11 +2,13 @@
 without a contact test may never hide a contact, also where the margin (gap + noise)
 - thr (v - v_L) falls because the car slows (a negative threshold: uphill, drag) or
 because drag drives it (a negative air density).  Most samples of every model trigger;
-binary64 gives the oracle's bits."""
+binary64 gives the oracle's bits, binary32 stays within its bounds of it (no drag that
+drives: binary32 scales by the drag coefficient's root)."""
 import numpy as np
 import pytest
 
 import aeb_inputs as ai
+from fp32_bounds import fp32_report, resolve_onset_ties, with_gap
 
 pytestmark = pytest.mark.gpu
 
@@ -83,3 +85,19 @@ def test_fp64_triggers_as_the_oracle(aeb, oracle_mod, kind, copies):
             got, want = got.view(np.uint64), want.view(np.uint64)
         bad = np.nonzero(got != want)[0]
         assert len(bad) == 0, (k, len(bad), bad[:5])
+
+
+@pytest.mark.parametrize("kind", list(CASES))
+def test_fp32_triggers_within_bounds(aeb, oracle_mod, kind):
+    m = CASES[kind][0]
+    p = _params(CASES[kind], 4)
+    exp = oracle_mod.rollout(m, p, threads=8)
+    assert np.mean(exp["n_onset"] >= 0) > 0.5
+    P = {f: torch.from_numpy(np.ascontiguousarray(p[f])).cuda() for f in ai.FIELDS}
+    out = aeb.alloc_outputs(N)
+    aeb.aeb_rollout(m, P, N, aeb.FP32_COMP, out)
+    torch.cuda.synchronize()
+    got = {k: v.cpu().numpy() for k, v in out.items()}
+    exp, ties = resolve_onset_ties(oracle_mod, m, p, np.arange(N), got, exp)
+    fp32_report(m, with_gap(got, p, m), with_gap(exp, p, m), ties)
+    assert ties[0] <= 3, ties

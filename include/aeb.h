@@ -385,10 +385,12 @@ aeb_status aeb_reduce_weighted(const aeb_outputs *out, const double *weights, ui
  *   out        device columns (caller-owned; NULL members are skipped)
  *   stream     cudaStream_t
  * Asynchronous.  n == 0 is a no-op.
- * A launch of more than 32 samples in binary64, 19,456 in FP32, takes them in an
- * order of its own, kept in scratch of the library (6 B per sample, at most
- * 100 MB, allocated and freed on the stream); without that scratch, or while the stream is being
- * captured, in index order.  No output depends on the order.
+ * A launch of more than 32 samples in binary64, or in FP32 of more than 19,456
+ * with enough steps up to the horizon (1,000 to 3,000, and 1e8 to 4e8 samples times
+ * steps, by trigger, lead and size), takes them in an order of its own, kept in
+ * scratch of the library (6 B per sample, at most 100 MB, allocated and freed on
+ * the stream); without that scratch, or while the stream is being captured, in
+ * index order.  No output depends on the order.
  * AEB_EINVAL: NULL params column, bad model (non-finite constant, dt <= 0,
  * t_max < 0, t_max/dt beyond 2^31 - 2 steps, unknown mode, reserved != 0,
  * wheelbase <= 0), unknown precision, misaligned column.

@@ -104,7 +104,9 @@ cudaError_t launch_rollout_fp32(const ModelDev &m, const ParamsDev &p, const Out
 // host_tiles is the host copy of w.tiles.  `scratch` holds rollout_scratch_bytes
 // of the work's positions, or only kCounterBytes: then the order is natural.
 constexpr size_t kCounterBytes = 256;
-size_t rollout_scratch_bytes(uint64_t positions, aeb_precision precision);
+size_t rollout_scratch_bytes(uint64_t positions, aeb_precision precision, const ModelDev &m);
+// The same for launches of any size up to `positions`.
+size_t rollout_scratch_bytes_up_to(uint64_t positions, aeb_precision precision, const ModelDev &m);
 cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision precision,
                            const OutDev &o, const WorkDev &w, const TileDesc *host_tiles,
                            const LaunchCfg &cfg, void *scratch, size_t scratch_bytes,

@@ -102,7 +102,7 @@ aeb_status lay_out(const char *who, const aeb_model *model, const aeb_job *jobs,
     L->o_first = L->o_red + a256(sizeof(TileDesc) * L->red.size());
     L->o_part = L->o_first + a256(sizeof(uint32_t) * L->first.size());
     L->o_scratch = L->o_part + a256(sizeof(RedPartial) * (L->red.size() + 1));
-    L->scratch = rollout_scratch_bytes((uint64_t)L->tiles.size() * T, precision);
+    L->scratch = rollout_scratch_bytes((uint64_t)L->tiles.size() * T, precision, L->md);
     return AEB_OK;
 }
 

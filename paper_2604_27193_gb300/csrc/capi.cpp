@@ -255,7 +255,7 @@ aeb_status rollout_impl(const ModelDev &md, const ParamsDev &pd, uint64_t n,
     aeb_status st = scratch_for(s, kCounterBytes + partial_bytes(), &scratch);
     if (st != AEB_OK) return st;
     const LaunchCfg cfg = launch_cfg(precision);
-    const size_t want = rollout_scratch_bytes(n, precision);
+    const size_t want = rollout_scratch_bytes(n, precision, md);
     void *order = want > kCounterBytes ? pool_alloc(want, s) : nullptr;
     const WorkDev w{n, ticket_tile(cfg), nullptr, nullptr, 0, nullptr, key_base, 0, nullptr};
     cudaError_t e = launch_rollout(md, pd, precision, od, w, nullptr, cfg, order ? order : scratch,

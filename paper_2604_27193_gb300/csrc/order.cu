@@ -289,22 +289,65 @@ struct Layout {
     }
 };
 
-// Whether a launch of this many positions is worth ordering.  With at most
-// one warp per sub-partition (152 x 4 x 32 = 19,456 rollouts) a binary32 launch
-// lasts as long as its longest rollout in any order, and the two kernels would
-// add ~10 us to ~200.  A binary64 warp gains from lanes of one cap class at
-// any size above one warp (its steps take microseconds).
-bool wants_order(uint64_t positions, aeb_precision precision)
+// Whether a launch of this many positions is worth ordering.
+//
+// Binary64: a warp gains from lanes of one cap class at any size above one warp
+// (its steps take microseconds).
+//
+// Binary32: the two kernels and the clear cost ~13 us and 24 ns per 1,000
+// samples, and rows taken out of order cost more memory traffic; both have to come
+// back from steps.  Measured, ordered against index order, over 2e4 .. 1e7 samples
+// and horizons of 200 .. 10,000 steps (steps of 1 ms cut short, and whole 10 s
+// horizons of coarser steps):
+//   - at most one warp per sub-partition (152 x 4 x 32 = 19,456 rollouts) lasts as
+//     long as its longest rollout in any order;
+//   - below 1,000 steps: 1e6 samples of 200 steps 280 -> 314 us, of 500 572 -> 574,
+//     of 700 742 -> 712, of 1,000 995 -> 938; 1e7 of 700 coarse steps 4,021 -> 4,314,
+//     of 1,000 4,892 -> 4,818;
+//   - samples times steps: 1e8 and more pay (2e4 of 3,000 steps 150 -> 153 us, of
+//     5,000 219 -> 210; 4e4 of 2,000 134 -> 135, of 3,000 180 -> 172; 6e4 of 1,000
+//     coarse 66 -> 69, of 1,500 83 -> 81; 1e5 of 700 113 -> 115, of 1,000 142 -> 139);
+//   - without a lead, a horizon of a few seconds ends every rollout at the same
+//     step and only the cap classes gain: 4e8 and 1,500 steps (1e5 of 3,000 steps
+//     284 -> 293 us, 2e5 of 2,000 340 -> 340, 4e5 of 1,500 477 -> 477, 1e6 of 1,000
+//     829 -> 836, of 1,500 1,176 -> 1,148; at 5 s 1e5 462 -> 450);
+//   - the TTC trigger reads two columns more per sample, which counts once the
+//     columns no longer stay in the L2: 5e5 and more samples take 2,000 steps (1e6
+//     of 1,000 coarse steps 1.05 of index order, of 1,500 0.96, of 2,000 0.89), 2e6
+//     and more 3,000 (1e7 of 2,000 1.03; 3e6 of 3,000 0.89);
+//   - per-step readings take time that the order does not save: 2e8 and 2,000 steps
+//     (4e4 of 3,000 coarse steps 1.01, of 5,000 0.99; 1e5 of 1,500 1.00, of 2,000 0.98).
+constexpr uint64_t kTtcMid = uint64_t(1) << 19, kTtcMany = uint64_t(1) << 21;
+bool wants_order(uint64_t positions, aeb_precision precision, const ModelDev &m)
 {
-    return positions > (precision == AEB_FP64_PLAIN ? 32u : 19456u);
+    if (m.n_max <= 0) return false;
+    if (precision == AEB_FP64_PLAIN) return positions > 32;
+    if (positions <= 19456) return false;
+    const bool ttc = m.trigger == AEB_TRIGGER_TTC, readings = ttc && m.perc;
+    const bool cut = !m.lead && m.n_max * m.dt < 4.0;
+    const int32_t steps = ttc && positions > kTtcMany               ? 3000
+                          : readings || (ttc && positions > kTtcMid) ? 2000
+                          : cut                                      ? 1500
+                                                                     : 1000;
+    const double work = cut ? 4e8 : readings ? 2e8 : 1e8;
+    return m.n_max >= steps && (double)positions * m.n_max >= work;
 }
+
+size_t order_bytes(uint64_t positions) { return Layout(std::min(positions, kOrderMax)).bytes; }
 
 }  // namespace
 
-size_t rollout_scratch_bytes(uint64_t positions, aeb_precision precision)
+size_t rollout_scratch_bytes(uint64_t positions, aeb_precision precision, const ModelDev &m)
 {
-    if (!wants_order(positions, precision)) return kCounterBytes;
-    return Layout(std::min(positions, kOrderMax)).bytes;
+    return wants_order(positions, precision, m) ? order_bytes(positions) : kCounterBytes;
+}
+
+size_t rollout_scratch_bytes_up_to(uint64_t positions, aeb_precision precision, const ModelDev &m)
+{
+    // (the rule asks for more steps above kTtcMid and kTtcMany, otherwise for fewer)
+    for (const uint64_t most : {positions, kTtcMany, kTtcMid})
+        if (most <= positions && wants_order(most, precision, m)) return order_bytes(most);
+    return kCounterBytes;
 }
 
 cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision precision,
@@ -313,8 +356,7 @@ cudaError_t launch_rollout(const ModelDev &m, const ParamsDev &p, aeb_precision 
                            cudaStream_t s)
 {
     const uint64_t all = w.tiles ? w.n_tiles * w.tile : w.n;
-    const bool order = m.n_max > 0 && wants_order(all, precision) &&
-                       scratch_bytes >= rollout_scratch_bytes(all, precision);
+    const bool order = wants_order(all, precision, m) && scratch_bytes >= order_bytes(all);
     const uint64_t piece = order ? kOrderMax : kNaturalMax;  // positions per launch
     const uint64_t unit = w.tiles ? piece / w.tile : piece;   // tiles or rows per launch
     const uint64_t total = w.tiles ? w.n_tiles : w.n;

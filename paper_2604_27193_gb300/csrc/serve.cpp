@@ -618,7 +618,7 @@ extern "C" aeb_status aeb_serve_create(const aeb_serve_cfg *cfg, const aeb_model
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming);
         const size_t tables = sz_jobs + sz_tiles + sz_red + sz_first + sz_part + sz_stats;
         if (e == cudaSuccess) {
-            w.scratch_bytes = rollout_scratch_bytes(max_tiles * T, cfg->precision);
+            w.scratch_bytes = rollout_scratch_bytes_up_to(max_tiles * T, cfg->precision, md);
             e = cudaMalloc(&w.dmem, tables + w.scratch_bytes);
             if (e == cudaErrorMemoryAllocation && w.scratch_bytes > kCounterBytes) {
                 cudaGetLastError();

@@ -75,21 +75,16 @@ struct WorkDev {
 struct LaunchCfg {
     int block;          // threads per block (multiple of 32)
     int blocks_per_sm;  // resident blocks per SM requested (0: occupancy max)
-    int tile;           // samples per tile (multiple of 32)
-    bool tile_set;      // the tile was chosen by the caller or the autotuner
+    int tile;           // samples per ticket (multiple of 32)
 };
 
-// Samples a warp takes per ticket.  Unless a caller chose the tile it is one
-// warp's width in both precisions: a binary64 step costs a warp 64 cycles per
+// Samples a warp takes per ticket, unless a caller or the autotuner chooses:
+// one warp's width in both precisions.  A binary64 step costs a warp 64 cycles per
 // operation however few of its lanes are busy, so a small launch must spread
 // over as many warps as it can fill (1e4 binary64 rollouts: 87.8 ms in tiles of
 // 256, 17.1 ms in tiles of 32; 2.5e5: 157 and 146 ms), and one ticket per 32
 // rollouts costs nothing beside their steps.
 constexpr int kTicketSamples = 32;
-inline uint32_t ticket_tile(const LaunchCfg &c)
-{
-    return (uint32_t)(c.tile_set ? c.tile : kTicketSamples);
-}
 
 // Launchers of one kernel (asynchronous on `stream`; return a cudaError_t of
 // the launch).

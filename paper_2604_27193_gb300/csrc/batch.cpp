@@ -81,7 +81,7 @@ aeb_status lay_out(const char *who, const aeb_model *model, const aeb_job *jobs,
     if (reinterpret_cast<uintptr_t>(stats) % 8 != 0)
         return fail(AEB_EINVAL, w + ": stats is not 8-byte aligned");
     L->cfg = launch_cfg(precision);
-    const uint32_t T = L->T = ticket_tile(L->cfg);
+    const uint32_t T = L->T = (uint32_t)L->cfg.tile;
     L->jobs.resize(n_jobs);
     L->first.resize(n_jobs + 1);
     for (uint32_t j = 0; j < n_jobs; ++j) {
@@ -267,7 +267,6 @@ extern "C" aeb_status aeb_set_launch_config(aeb_precision precision, const aeb_l
     LaunchCfg c = launch_cfg(precision);
     c.tile = cfg->tile;
     c.blocks_per_sm = cfg->blocks_per_sm;
-    c.tile_set = true;
     set_launch_cfg(precision, c);
     return AEB_OK;
 }
@@ -350,7 +349,6 @@ extern "C" aeb_status aeb_autotune(const aeb_model *model, const aeb_params *par
             LaunchCfg c = saved;
             c.tile = tl[ti];
             c.blocks_per_sm = bps;
-            c.tile_set = true;
             set_launch_cfg(precision, c);
             float ms = 0.0f;
             for (int rep = 0; rep < 2 && st == AEB_OK; ++rep) {  // warm-up, then timed

@@ -245,7 +245,7 @@ void *pool_alloc(size_t bytes, cudaStream_t s)
 namespace {
 
 std::mutex g_cfg_mu;
-LaunchCfg g_cfg[2] = {{128, 0, 256, false}, {128, 0, 32, false}};
+LaunchCfg g_cfg[2] = {{128, 0, kTicketSamples}, {128, 0, kTicketSamples}};
 
 aeb_status rollout_impl(const ModelDev &md, const ParamsDev &pd, uint64_t n,
                         aeb_precision precision, const OutDev &od, cudaStream_t s,
@@ -257,7 +257,7 @@ aeb_status rollout_impl(const ModelDev &md, const ParamsDev &pd, uint64_t n,
     const LaunchCfg cfg = launch_cfg(precision);
     const size_t want = rollout_scratch_bytes(n, precision, md);
     void *order = want > kCounterBytes ? pool_alloc(want, s) : nullptr;
-    const WorkDev w{n, ticket_tile(cfg), nullptr, nullptr, 0, nullptr, key_base, 0, nullptr};
+    const WorkDev w{n, (uint32_t)cfg.tile, nullptr, nullptr, 0, nullptr, key_base, 0, nullptr};
     cudaError_t e = launch_rollout(md, pd, precision, od, w, nullptr, cfg, order ? order : scratch,
                                    order ? want : kCounterBytes, s);
     if (order) {

@@ -369,7 +369,7 @@ bool aeb_server::launch_wave(Wave &w)
     }
     if (w.chunks.empty()) return false;
     for (auto &c : w.chunks) c.req->inflight++;
-    const uint32_t T = ticket_tile(lcfg);
+    const uint32_t T = (uint32_t)lcfg.tile;
     const uint32_t nj = (uint32_t)w.chunks.size();
     uint32_t nt = 0, nr = 0;
     for (uint32_t j = 0; j < nj; ++j) {
@@ -603,7 +603,7 @@ extern "C" aeb_status aeb_serve_create(const aeb_serve_cfg *cfg, const aeb_model
     s->wave_timeout_ms = cfg->wave_timeout_ms == 0 ? kDefaultWaveTimeoutMs : cfg->wave_timeout_ms;
     e = cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking);
     // wave slots
-    const uint64_t T = ticket_tile(s->lcfg);
+    const uint64_t T = (uint64_t)s->lcfg.tile;
     const uint64_t max_tiles = cfg->wave_samples / T + kMaxJobsPerWave;
     const uint64_t max_red = cfg->wave_samples / kRedSegment + kMaxJobsPerWave;
     const size_t sz_jobs = a256(sizeof(JobDev) * kMaxJobsPerWave);

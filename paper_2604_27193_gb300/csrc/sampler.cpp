@@ -9,6 +9,7 @@
 // library's idle sampling threads take [0, n) in pieces of kGrain samples.  Built with -ffp-contract=off so the binary64 transforms
 // round the same on every host.
 #include <pthread.h>
+#include <sched.h>
 
 #include <algorithm>
 #include <atomic>
@@ -181,7 +182,8 @@ constexpr uint64_t kGrain = 256;
 // started when a call first wants them (one fewer than the host's threads), wait
 // for work and end after a second without any.  The calling thread works too
 // and only waits for pieces a helper has begun, so a call never depends on a
-// helper being there.
+// helper being there.  A helper runs on the CPUs of the call it helps (as a thread
+// that the call had started would), not on those of the call that started it.
 class Workers {
   public:
     using Piece = std::function<void(uint64_t, uint64_t)>;
@@ -205,6 +207,7 @@ class Workers {
         const unsigned helpers =
             (unsigned)std::min<uint64_t>({job.max_helpers, pieces - 1, max_threads_});
         if (helpers > 0) {
+            job.note_cpus();
             std::lock_guard<std::mutex> lk(mu_);
             jobs_.push_back(&job);
             while (idle_ + starting_ < helpers && threads_ < max_threads_) {
@@ -233,7 +236,13 @@ class Workers {
         const unsigned max_helpers;
         std::atomic<uint64_t> next{0};
         unsigned helpers = 0;  // threads inside take(), under the pool's lock
+        cpu_set_t cpus;        // of the calling thread (cpus_known)
+        bool cpus_known = false;
         Job(uint64_t n_, const Piece *f_, unsigned m) : n(n_), f(f_), max_helpers(m) {}
+        void note_cpus()
+        {
+            cpus_known = pthread_getaffinity_np(pthread_self(), sizeof cpus, &cpus) == 0;
+        }
         void take()
         {
             for (uint64_t lo; (lo = next.fetch_add(kGrain)) < n;)
@@ -249,6 +258,8 @@ class Workers {
 
     void loop()
     {
+        cpu_set_t mine;
+        bool known = pthread_getaffinity_np(pthread_self(), sizeof mine, &mine) == 0;
         std::unique_lock<std::mutex> lk(mu_);
         --starting_;
         for (;;) {
@@ -270,6 +281,10 @@ class Workers {
             }
             ++job->helpers;
             lk.unlock();
+            if (job->cpus_known && !(known && CPU_EQUAL(&mine, &job->cpus))) {
+                mine = job->cpus;
+                known = pthread_setaffinity_np(pthread_self(), sizeof mine, &mine) == 0;
+            }
             job->take();
             lk.lock();
             if (--job->helpers == 0) done_.notify_all();  // the job may be gone after this

@@ -81,7 +81,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
             if log.strip():
                 print(log, file=sys.stderr)
     tmp = LIB + f".tmp{os.getpid()}"
-    _run([NVCC, *ARCH, "-shared", "-o", tmp, *[o for _, o in jobs], "-lpthread"])
+    # (never unmapped: the sampler's idle threads outlive a call by up to a second,
+    # and code they return into must still be there after a dlclose)
+    _run([NVCC, *ARCH, "-shared", "-Xlinker", "-z", "-Xlinker", "nodelete", "-o", tmp,
+          *[o for _, o in jobs], "-lpthread"])
     os.replace(tmp, LIB)
     return LIB
 

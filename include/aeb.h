@@ -17,8 +17,13 @@
  * Conventions for every entry point:
  *   - Plain C types only; pointers are host or device as each argument says.
  *   - Buffers passed in are owned by the caller and never freed or retained by
- *     the library after the call's stream work completes.  Library-owned
- *     scratch is allocated on first use per device and reused.
+ *     the library after the call's stream work completes.  Counters, partial
+ *     sums and the buffers of aeb_evaluate (which grow to its largest call)
+ *     are allocated on first use per device and stream and reused.  The order
+ *     of a rollout, the tables of a one-shot batch and the buffers of a sweep
+ *     come from a memory pool of the library per device, allocated and freed
+ *     in stream order in each call; up to 256 MB stay with the pool between
+ *     calls.
  *   - `stream` is a cudaStream_t (NULL = legacy default stream).  Calls marked
  *     "asynchronous" only enqueue work on it; results are valid once the
  *     stream has reached that point.
@@ -328,8 +333,13 @@ const char *aeb_last_error(void);
  * U2 = (w1>>11) 2^-53.  Then clamp.  gs, gc = g sin(grade), g cos(grade).
  *   model    host; only model->g is read
  *   out      host columns (caller-owned, >= n doubles each)
- *   n_threads host threads to use (<= 0: all hardware threads)
+ *   n_threads host threads to use, the caller's included (<= 0: all hardware
+ *            threads; never more than those)
  * Synchronous, host only.  Output is independent of n_threads.
+ * The threads that help are the library's own, shared by every call that
+ * samples: started when a call wants them, on the CPUs of the call they help,
+ * ended after a second without work.  The library is marked to stay loaded
+ * (a dlclose does not unmap it).
  * AEB_EINVAL: NULL pointer, unknown distribution kind, non-finite parameter.
  */
 aeb_status aeb_sample_params(const aeb_model *model, const aeb_scenario *scenario,
@@ -486,9 +496,10 @@ aeb_status aeb_evaluate_scenario(const aeb_model *model, const aeb_scenario *sce
  * aeb_batch_create -- plan a batched launch over n_jobs jobs (the per-sample
  * method is that of aeb_rollout, Sec. IV-D, V-A..V-D).  Builds
  * the table of (job, tile) work items, allocates the device tables and
- * scratch (owned by the plan), and captures one CUDA graph: reset of the work
- * counter, one persistent rollout launch over all tiles, and the per-job
- * fixed-order reduction into stats[0 .. n_jobs).
+ * scratch (owned by the plan; with those of an order, see aeb_rollout, 6 B per
+ * sample and at most 100 MB more), and captures one CUDA graph: reset of the
+ * work counter, the order's kernels, a persistent rollout launch over all
+ * tiles, and the per-job fixed-order reduction into stats[0 .. n_jobs).
  *   jobs       host array (copied)
  *   params     device columns (caller-owned; must outlive the plan)
  *   out        device output columns covering every job's out rows; status,
@@ -510,8 +521,10 @@ aeb_status aeb_batch_run(aeb_batch *plan, void *stream);
 void aeb_batch_destroy(aeb_batch *plan);
 
 /*
- * aeb_rollout_batched -- create, run once on `stream` and destroy a plan
- * (synchronous: returns when the stats are written).
+ * aeb_rollout_batched -- what a plan of these jobs does, once, on `stream`
+ * (synchronous: returns when the stats are written).  Builds no graph and takes
+ * its device tables and scratch from the library's pool; a plan is created, run
+ * and destroyed only where the pool has no memory.
  */
 aeb_status aeb_rollout_batched(const aeb_model *model, const aeb_job *jobs, uint32_t n_jobs,
                                const aeb_params *params, aeb_precision precision,
@@ -544,8 +557,9 @@ aeb_status aeb_autotune(const aeb_model *model, const aeb_params *params, uint64
  * persistent launch each; consecutive waves overlap on two streams).  A
  * request's statistics are the fixed-order combination of its chunks' and do
  * not depend on what it shares waves with.
- * Allocates the arena, pinned staging and wave buffers, and starts two host
- * threads.  AEB_EINVAL on a bad configuration, AEB_ENOMEM if the arena cannot
+ * Allocates the arena, pinned staging and wave buffers (per wave in flight its
+ * tables and, for the order of its rollouts, up to 6 B per wave sample), and
+ * starts two host threads.  AEB_EINVAL on a bad configuration, AEB_ENOMEM if the arena cannot
  * be allocated.
  */
 aeb_status aeb_serve_create(const aeb_serve_cfg *cfg, const aeb_model *model, aeb_server **out);
@@ -600,8 +614,9 @@ void aeb_serve_destroy(aeb_server *srv);
  * model->trigger forced to AEB_TRIGGER_TTC.
  *   per_threshold  host, n_thr entries: pooled counts, p, Wilson 95 % interval
  *   per_job        host, n_thr * n_scen entries (threshold-major) or NULL
- * Synchronous; allocates and frees its device buffers (about
- * 80 B x n_scen x n_per_scenario for parameters plus up to 4.5 GB of outputs).
+ * Synchronous; its device buffers (about 80 B x n_scen x n_per_scenario for
+ * parameters plus up to 4.5 GB of outputs) come from the library's pool and go
+ * back to it.
  */
 aeb_status aeb_ttc_sweep(const aeb_model *model, const aeb_scenario *scenarios, uint32_t n_scen,
                          uint64_t n_per_scenario, const double *thresholds, uint32_t n_thr,

@@ -22,8 +22,9 @@
 //
 // Two kernels before the rollouts: bin every position by (cap class, length,
 // turn), then scatter the positions to their bins' ranges (a counting sort; the
-// order inside a bin is free).  72 B read and 8 B written and read per
-// sample.
+// order inside a bin is free).  Per sample 56 B of columns read (64 B with a
+// lead, 72 B with the TTC trigger), a 2-byte key and a 4-byte position written
+// and read.
 #include <algorithm>
 #include <cmath>
 

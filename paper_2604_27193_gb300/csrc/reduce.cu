@@ -7,7 +7,7 @@
 //   strided share in index order and queues the values that enter a sum (D_stop
 //   of a stop, the impact speed of a contact) by kind in shared memory; 32
 //   queued values of a kind are then summed, compared and binned together, so
-//   the binary64 unit, which holds a warp instruction 64 cycles whatever its
+//   the binary64 unit, which a warp instruction holds 64 cycles or more whatever its
 //   busy lanes, is paid once per 32 values instead of once per kind and 32
 //   samples.  The block combines its lanes in a fixed order into one partial.
 //   Histogram bins are counted with shared-memory atomics and flushed with 64-bit global
@@ -193,9 +193,12 @@ struct RedShared {
 };
 static_assert(sizeof(RedShared) + 8 * AEB_NBINS <= 96 * 1024, "two blocks per SM");
 
-// SHIFT: an origin of the histograms is not 0 (without one the subtraction, a
-// third binary64 operation per 32 values, is left out: x - 0 is x; 1e7 samples
-// 98 -> 78 us).
+// SHIFT: an origin of the histograms is not 0 (without one the subtraction is
+// left out: x - 0 is x; 1e7 samples 98 -> 78 us).
+// What bounds it: the binary64 unit, 76 % busy.  Counted without SHIFT: three warp
+// instructions of that unit per 32 values, one more than the two written, each
+// holding it 73 cycles (k_reduce_weighted: the two written, 77 cycles); the
+// rollout kernel's register forms take 65.
 // HIST: accumulate the two histograms and let the last block finish the
 // statistics (the count in stats->n, clear at launch, tells which one that is).
 // With a block table, block b reduces rows [out_offset + first, + count) of job

@@ -11,7 +11,7 @@
 // owns samples [b*chunk, (b+1)*chunk); a warp walks its strided share in index
 // order and queues the weights of events and of the other valid samples in shared
 // memory; 32 queued weights of a kind are then added together (the binary64 unit
-// holds a warp instruction 64 cycles whatever its busy lanes, so each weight
+// is held 64 cycles or more by a warp instruction whatever its busy lanes, so each weight
 // enters one pair of sums, not two; all = events + others).  The block adds its
 // threads with a fixed tree and writes one partial; the block that arrives last
 // adds the G partials with the same tree.  One pass over 17 bytes per sample
